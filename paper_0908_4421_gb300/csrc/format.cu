@@ -166,6 +166,8 @@ __device__ __forceinline__ void store_col(void* dst, int64_t k, int32_t c) {
 // One CTA per slice: thread o of the slice writes stored position o (group o / (32 GE), lane
 // (o / GE) % 32, place o % GE), so the writes are coalesced and a long row is spread over
 // the CTA instead of being walked by one thread (C16: 16-bit beamlet indices with FP32 values).
+// Bound by HBM once loads are in flight: a thread's kU positions are all loaded before any is
+// stored (61M entries to FP32 / FP16: 0.30 / 0.32 -> 0.16 / 0.17 ms, 0.13 ms at the copy rate).
 template <int PREC, int GE, bool C16 = false>
 __global__ void __launch_bounds__(256) k_sell_fill(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                                                    const float* __restrict__ val, const int32_t* __restrict__ perm,
@@ -187,20 +189,28 @@ __global__ void __launch_bounds__(256) k_sell_fill(const int64_t* __restrict__ r
     }
     __syncthreads();
     const int64_t base = slice_off[s];
-    const int64_t total = (int64_t)slice_len[s] * GE * kSlice;
-    for (int64_t o = threadIdx.x; o < total; o += blockDim.x) {
-        const int within = (int)(o % (kSlice * GE));
-        const int lane = within / GE;
-        const int e = (int)(o / (kSlice * GE)) * GE + within % GE;
-        if (e < rl[lane]) {
-            const int64_t k = ra[lane] + e;
-            const int c = col[k];
-            const float v = inv_scale ? val[k] * inv_scale[c] : val[k];
-            store_val<PREC>(sval, base + o, v);
-            store_col<PREC, C16>(scol, base + o, c);
-        } else {
-            store_val<PREC>(sval, base + o, 0.0f);
-            store_col<PREC, C16>(scol, base + o, 0);
+    const int total = slice_len[s] * GE * kSlice;
+    constexpr int kU = 8;
+    for (int o0 = threadIdx.x; o0 < total; o0 += kU * 256) {
+        int c[kU];
+        float v[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int o = o0 + u * 256;
+            const int within = o % (kSlice * GE);
+            const int lane = within / GE;
+            const int e = o / (kSlice * GE) * GE + within % GE;
+            const bool in = o < total && e < rl[lane];
+            c[u] = in ? __ldg(col + ra[lane] + e) : -1;  // -1: padding (value 0, column 0)
+            v[u] = in ? __ldg(val + ra[lane] + e) : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int o = o0 + u * 256;
+            if (o < total) {
+                store_val<PREC>(sval, base + o, inv_scale && c[u] >= 0 ? v[u] * inv_scale[c[u]] : v[u]);
+                store_col<PREC, C16>(scol, base + o, max(c[u], 0));
+            }
         }
     }
 }
@@ -228,24 +238,53 @@ __global__ void k_t_count(const int64_t* __restrict__ row_ptr, const int32_t* __
     for (int c = threadIdx.x; c < n; c += blockDim.x) counts[(size_t)blockIdx.x * n + c] = hist[c];
 }
 
-// Pass 2: per beamlet, exclusive offsets of each chunk inside the beamlet's row; totals.
-__global__ void k_t_colscan(int32_t* __restrict__ counts, int32_t n_chunks, int32_t n, int64_t* __restrict__ col_len,
-                            int64_t* __restrict__ padded) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+// Pass 2: per beamlet, exclusive offsets of each chunk inside the beamlet's row; totals. A block takes
+// 32 beamlets (coalesced counts); its kScanParts rows of threads each take a run of chunks, first
+// added up, then written as offsets from the scan of the runs' sums (one thread a beamlet over all chunks
+// was a serial chain of round trips: 82 us for 596 chunks, now 24 us for 2382).
+constexpr int kScanParts = 32;
+__global__ void __launch_bounds__(32 * kScanParts) k_t_colscan(int32_t* __restrict__ counts, int32_t n_chunks, int32_t n,
+                                                              int64_t* __restrict__ col_len,
+                                                              int64_t* __restrict__ padded) {
+    __shared__ int32_t part[kScanParts][33];
+    const int lane = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int c = blockIdx.x * 32 + lane;
+    const int per = (n_chunks + kScanParts - 1) / kScanParts;
+    const int ch0 = min(n_chunks, y * per), ch1 = min(n_chunks, ch0 + per);
+    constexpr int kU = 8;  // loads in flight
+    int sum = 0;
+    if (c < n) {
+        for (int ch = ch0; ch < ch1; ch += kU) {
+            int v[kU];
+#pragma unroll
+            for (int t = 0; t < kU; ++t) v[t] = ch + t < ch1 ? counts[(size_t)(ch + t) * n + c] : 0;
+#pragma unroll
+            for (int t = 0; t < kU; ++t) sum += v[t];
+        }
+    }
+    part[y][lane] = sum;
+    __syncthreads();
+    int run = 0, total = 0;
+    for (int k = 0; k < kScanParts; ++k) {
+        const int v = part[k][lane];
+        run += k < y ? v : 0;
+        total += v;
+    }
     if (c >= n) return;
-    int64_t run = 0;
-    for (int ch0 = 0; ch0 < n_chunks; ch0 += 8) {  // eight loads in flight per step
-        int v[8];
+    if (y == 0) {
+        col_len[c] = total;
+        padded[c] = ((int64_t)total + 3) & ~(int64_t)3;
+    }
+    for (int ch = ch0; ch < ch1; ch += kU) {
+        int v[kU];
 #pragma unroll
-        for (int t = 0; t < 8; ++t) v[t] = ch0 + t < n_chunks ? counts[(size_t)(ch0 + t) * n + c] : 0;
+        for (int t = 0; t < kU; ++t) v[t] = ch + t < ch1 ? counts[(size_t)(ch + t) * n + c] : 0;
 #pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            if (ch0 + t < n_chunks) counts[(size_t)(ch0 + t) * n + c] = (int32_t)run;
+        for (int t = 0; t < kU; ++t) {
+            if (ch + t < ch1) counts[(size_t)(ch + t) * n + c] = run;
             run += v[t];
         }
     }
-    col_len[c] = run;
-    padded[c] = (run + 3) & ~(int64_t)3;
 }
 
 // Pass 3: scatter. Rows of a chunk are visited in order, so each beamlet row
@@ -383,36 +422,60 @@ __global__ void k_tq_count(const int64_t* __restrict__ t_off, const int32_t* __r
     }
 }
 
+// The segmented copy of beamlet row i, one CTA a row, and with PREC != FP32 the reduced copy of the same
+// places beside it. A thread makes one group of 8 stored entries: group l of a piece of sg groups holds
+// the run's entries l, l + sg, ..., l + 7 sg (kTqBlock), so a warp's reads are consecutive entries of the
+// row and its writes whole 16-byte words. 61M entries, FP32 + FP16: 0.17 ms (0.14 ms at the copy rate);
+// one thread an entry, with a division by sg for its place, and a launch a copy took 0.40 + 0.34 ms.
 template <int PREC>
-__global__ void k_tq_fill(const int64_t* __restrict__ t_off, const int32_t* __restrict__ t_row,
-                          const float* __restrict__ t_val, const int64_t* __restrict__ col_len, int32_t n, int32_t H,
-                          const int64_t* __restrict__ seg, const float* __restrict__ inv_scale, void* q_val,
-                          uint16_t* __restrict__ q_lo) {
+__global__ void __launch_bounds__(256) k_tq_fill(const int64_t* __restrict__ t_off, const int32_t* __restrict__ t_row,
+                                                 const float* __restrict__ t_val, const int64_t* __restrict__ col_len,
+                                                 int32_t n, int32_t H, const int64_t* __restrict__ seg,
+                                                 const float* __restrict__ inv_scale, float* __restrict__ s_val,
+                                                 void* q_val, uint16_t* __restrict__ q_lo) {
+    __shared__ int64_t sb[kMaxSegments + 1];   // first stored entry of each segment, and the row's end
+    __shared__ int64_t src[kMaxSegments + 1];  // first entry of each segment in the sorted row, and its end
     const int i = blockIdx.x;
-    if (i >= n) return;
     const int64_t a = t_off[i], b = a + col_len[i];
-    const int64_t r0 = seg[(int64_t)i * H];
-    const float s = inv_scale ? inv_scale[i] : 1.0f;
-    for (int h = 0; h < H; ++h) {
-        const int64_t lo_b = lower_bound_row(t_row, a, b, h << 16);
-        const int64_t hi_b = h + 1 < H ? lower_bound_row(t_row, a, b, (h + 1) << 16) : b;
-        const int64_t dst0 = seg[(int64_t)i * H + h], dst1 = seg[(int64_t)i * H + h + 1];
-        for (int64_t k = dst0 + threadIdx.x; k < dst1; k += blockDim.x) {
-            // k is the entry's place in the sorted run; it is stored at its transposed place
-            // inside the piece of its 256-entry block that lies in this run (all multiples of 8)
-            const int64_t blk = r0 + ((k - r0) & ~(int64_t)(kTqBlock - 1));
-            const int64_t ps = blk > dst0 ? blk : dst0;
-            const int64_t pe = blk + kTqBlock < dst1 ? blk + kTqBlock : dst1;
-            const int sg = (int)((pe - ps) >> 3), u = (int)(k - ps);
-            const int64_t d = ps + 8 * (u % sg) + u / sg;
-            const int64_t src = lo_b + (k - dst0);
-            if (src < hi_b) {
-                store_val<PREC>(q_val, d, t_val[src] * s);
-                q_lo[d] = (uint16_t)(t_row[src] & 0xffff);
-            } else {
-                store_val<PREC>(q_val, d, 0.0f);
-                q_lo[d] = 0;
-            }
+    if (threadIdx.x <= H) {
+        const int h = threadIdx.x;
+        sb[h] = seg[(int64_t)i * H + h];
+        src[h] = h == 0 ? a : h == H ? b : lower_bound_row(t_row, a, b, h << 16);
+    }
+    __syncthreads();
+    const int64_t r0 = sb[0];
+    const int groups = (int)((sb[H] - r0) >> 3);
+    const float s = PREC != IMRT_FP32 ? inv_scale[i] : 1.0f;
+    for (int k = threadIdx.x; k < groups; k += 256) {
+        const int64_t e = r0 + 8 * (int64_t)k;
+        int h = 0;
+        while (h + 1 < H && e >= sb[h + 1]) ++h;
+        const int64_t blk = r0 + ((e - r0) & ~(int64_t)(kTqBlock - 1));
+        const int64_t ps = blk > sb[h] ? blk : sb[h];
+        const int64_t pe = blk + kTqBlock < sb[h + 1] ? blk + kTqBlock : sb[h + 1];
+        const int sg = (int)((pe - ps) >> 3);
+        const int64_t f = src[h] + (ps - sb[h]) + ((e - ps) >> 3);
+        float v[8];
+        uint32_t lo[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const bool in = f + t * sg < src[h + 1];
+            v[t] = in ? __ldg(t_val + f + t * sg) : 0.0f;
+            lo[t] = in ? (uint32_t)__ldg(t_row + f + t * sg) & 0xffffu : 0u;
+        }
+        float4* sv = reinterpret_cast<float4*>(s_val + e);
+        sv[0] = make_float4(v[0], v[1], v[2], v[3]);
+        sv[1] = make_float4(v[4], v[5], v[6], v[7]);
+        *reinterpret_cast<uint4*>(q_lo + e) =
+            make_uint4(lo[0] | lo[1] << 16, lo[2] | lo[3] << 16, lo[4] | lo[5] << 16, lo[6] | lo[7] << 16);
+        if constexpr (PREC != IMRT_FP32) {
+            constexpr int kBytes = PREC == IMRT_FP8E4M3 ? 8 : 16;
+            __align__(16) unsigned char q[16];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) store_val<PREC>(q, t, f + t * sg < src[h + 1] ? v[t] * s : 0.0f);
+            unsigned char* dst = static_cast<unsigned char*>(q_val) + e * (kBytes / 8);
+            if constexpr (kBytes == 16) *reinterpret_cast<uint4*>(dst) = *reinterpret_cast<const uint4*>(q);
+            else *reinterpret_cast<uint2*>(dst) = *reinterpret_cast<const uint2*>(q);
         }
     }
 }
@@ -489,11 +552,27 @@ __global__ void __launch_bounds__(256) k_sum_masked_part(const float* __restrict
     if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-__global__ void k_col_absmax(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                             const float* __restrict__ val, int32_t m, uint32_t* __restrict__ absmax_bits) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= m) return;
-    for (int64_t k = row_ptr[j]; k < row_ptr[j + 1]; ++k) atomicMax(&absmax_bits[col[k]], __float_as_uint(fabsf(val[k])));
+// max |D_ij| of each beamlet, one CTA a row of the beamlet-major copy (coalesced: 43 us for
+// 61M entries, 36 at the copy rate; one thread a voxel row with an atomic maximum per entry took 3.1 ms).
+__global__ void __launch_bounds__(256) k_row_absmax(const int64_t* __restrict__ t_off, const int64_t* __restrict__ col_len,
+                                                    const float* __restrict__ t_val, uint32_t* __restrict__ absmax_bits) {
+    __shared__ uint32_t sh[8];
+    const int i = blockIdx.x;
+    const int64_t a = t_off[i], b = a + col_len[i];
+    uint32_t most = 0u;
+    constexpr int kU = 8;
+    for (int64_t k = a + threadIdx.x; k < b; k += kU * 256) {
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            most = max(most, k + u * 256 < b ? __float_as_uint(fabsf(__ldg(t_val + k + u * 256))) : 0u);
+    }
+    most = __reduce_max_sync(0xffffffffu, most);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = most;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) most = max(most, sh[w]);
+        absmax_bits[i] = most;
+    }
 }
 
 __global__ void k_scales(const uint32_t* __restrict__ absmax_bits, int32_t n, int32_t n_pad, float qmax,
@@ -597,7 +676,7 @@ cudaError_t launch_transpose_plan(const int64_t* row_ptr, const int32_t* col, in
         if (e != cudaSuccess) return e;
     }
     k_t_count<<<n_chunks, 256, smem, stream>>>(row_ptr, col, m, n, chunk_rows, counts);
-    k_t_colscan<<<blocks_for(n, 256), 256, 0, stream>>>(counts, n_chunks, n, col_len, padded);
+    k_t_colscan<<<blocks_for(n, 32), 32 * kScanParts, 0, stream>>>(counts, n_chunks, n, col_len, padded);
     k_scan_i64<<<1, 1024, 0, stream>>>(padded, t_off, n);
     return cudaGetLastError();
 }
@@ -635,20 +714,23 @@ cudaError_t launch_tq_count(const int64_t* t_off, const int32_t* t_row, const in
 
 cudaError_t launch_tq_fill(int precision, const int64_t* t_off, const int32_t* t_row, const float* t_val,
                            const int64_t* col_len, int32_t n, int32_t H, const int64_t* seg, const float* inv_scale,
-                           void* q_val, uint16_t* q_lo, cudaStream_t stream) {
+                           float* s_val, void* q_val, uint16_t* q_lo, cudaStream_t stream) {
     switch (precision) {
-        case IMRT_FP32:  // unscaled FP32 values in the segmented layout
-            k_tq_fill<IMRT_FP32><<<n, 256, 0, stream>>>(t_off, t_row, t_val, col_len, n, H, seg, nullptr, q_val, q_lo);
+        case IMRT_FP32:
+            k_tq_fill<IMRT_FP32><<<n, 256, 0, stream>>>(t_off, t_row, t_val, col_len, n, H, seg, inv_scale, s_val, q_val,
+                                                        q_lo);
             break;
         case IMRT_FP16:
-            k_tq_fill<IMRT_FP16><<<n, 256, 0, stream>>>(t_off, t_row, t_val, col_len, n, H, seg, inv_scale, q_val, q_lo);
+            k_tq_fill<IMRT_FP16><<<n, 256, 0, stream>>>(t_off, t_row, t_val, col_len, n, H, seg, inv_scale, s_val, q_val,
+                                                        q_lo);
             break;
         case IMRT_BF16:
-            k_tq_fill<IMRT_BF16><<<n, 256, 0, stream>>>(t_off, t_row, t_val, col_len, n, H, seg, inv_scale, q_val, q_lo);
+            k_tq_fill<IMRT_BF16><<<n, 256, 0, stream>>>(t_off, t_row, t_val, col_len, n, H, seg, inv_scale, s_val, q_val,
+                                                        q_lo);
             break;
         case IMRT_FP8E4M3:
-            k_tq_fill<IMRT_FP8E4M3><<<n, 256, 0, stream>>>(t_off, t_row, t_val, col_len, n, H, seg, inv_scale, q_val,
-                                                          q_lo);
+            k_tq_fill<IMRT_FP8E4M3><<<n, 256, 0, stream>>>(t_off, t_row, t_val, col_len, n, H, seg, inv_scale, s_val,
+                                                           q_val, q_lo);
             break;
         default:
             return cudaErrorInvalidValue;
@@ -705,9 +787,9 @@ cudaError_t launch_sum_masked(const float* z, const uint8_t* mask, int32_t bit, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_col_absmax(const int64_t* row_ptr, const int32_t* col, const float* val, int32_t m, int32_t,
+cudaError_t launch_row_absmax(const int64_t* t_off, const int64_t* col_len, const float* t_val, int32_t n,
                               uint32_t* absmax_bits, cudaStream_t stream) {
-    k_col_absmax<<<blocks_for(m, 256), 256, 0, stream>>>(row_ptr, col, val, m, absmax_bits);
+    k_row_absmax<<<n, 256, 0, stream>>>(t_off, col_len, t_val, absmax_bits);
     return cudaGetLastError();
 }
 

@@ -49,6 +49,7 @@ constexpr int kMaxPrefetchPerCta = 8;  // forward CTA's L2 prefetch targets (tra
 // Beamlet-major build: voxel rows per counting-sort chunk (doubled while the chunk x beamlet
 // count table would exceed kTCountBytes).
 constexpr int kTChunkRows = 512;
+constexpr int kMaxSegments = 16;  // of 65536 voxels, in a segmented beamlet-major copy
 constexpr int64_t kTCountBytes = 256ll << 20;
 constexpr int kCtlThreads = 256;
 constexpr int kTmaMaxConsumers = 8;   // bulk-copy forward kernel: 1 producer + up to 8 consumer warps
@@ -349,9 +350,11 @@ cudaError_t launch_transpose_fill(const int64_t* row_ptr, const int32_t* col, co
                                   const int64_t* t_off, float* t_val, int32_t* t_row, cudaStream_t stream);
 cudaError_t launch_tq_count(const int64_t* t_off, const int32_t* t_row, const int64_t* col_len, int32_t n, int32_t H,
                             int64_t* seg_len, cudaStream_t stream);
+// The FP32 segmented copy (s_val, q_lo) and, for a reduced precision, its scaled values in the same places
+// (q_val; NULL with IMRT_FP32).
 cudaError_t launch_tq_fill(int precision, const int64_t* t_off, const int32_t* t_row, const float* t_val,
                            const int64_t* col_len, int32_t n, int32_t H, const int64_t* seg, const float* inv_scale,
-                           void* q_val, uint16_t* q_lo, cudaStream_t stream);
+                           float* s_val, void* q_val, uint16_t* q_lo, cudaStream_t stream);
 cudaError_t launch_mask_counts(const uint8_t* mask, int32_t m, int32_t* counts, cudaStream_t stream);
 cudaError_t launch_unpermute(const float* zp, const int32_t* perm, int32_t m, float* z, cudaStream_t stream);
 cudaError_t launch_pad_copy(const float* src, int32_t n, int32_t n_pad, float* dst, cudaStream_t stream);
@@ -364,8 +367,9 @@ cudaError_t launch_sum_masked(const float* z, const uint8_t* mask, int32_t bit, 
                               double* scratch, cudaStream_t stream);
 cudaError_t launch_permute_in(const float* src, const uint8_t* src_mask, const int32_t* perm, int32_t m,
                               int32_t m_pad, float* dst, uint8_t* dst_mask, cudaStream_t stream);
-cudaError_t launch_col_absmax(const int64_t* row_ptr, const int32_t* col, const float* val, int32_t m,
-                              int32_t n, uint32_t* absmax_bits, cudaStream_t stream);
+// absmax_bits[i] = bits of max |D_ij| over row i of the beamlet-major copy (i < n).
+cudaError_t launch_row_absmax(const int64_t* t_off, const int64_t* col_len, const float* t_val, int32_t n,
+                              uint32_t* absmax_bits, cudaStream_t stream);
 cudaError_t launch_scales(const uint32_t* absmax_bits, int32_t n, int32_t n_pad, float qmax, float* scale,
                           float* inv_scale, cudaStream_t stream);
 cudaError_t launch_g_objective(const double* gpart, int32_t count, double* out, cudaStream_t stream);
