@@ -493,14 +493,6 @@ __global__ void k_mask_counts(const uint8_t* __restrict__ mask, int32_t m, int32
     if (threadIdx.x < kMaxStruct) atomicAdd(&counts[threadIdx.x], local[threadIdx.x]);
 }
 
-__global__ void k_unpermute(const float* __restrict__ zp, const int32_t* __restrict__ perm, int32_t m,
-                            float* __restrict__ z) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= m) return;
-    const int j = perm[p];
-    if (j >= 0) z[j] = zp[p];
-}
-
 // Caller order -> permuted order for per-voxel arrays (padding positions get 0).
 __global__ void k_permute_in(const float* __restrict__ src, const uint8_t* __restrict__ src_mask,
                              const int32_t* __restrict__ perm, int32_t m, int32_t m_pad, float* __restrict__ dst,
@@ -743,11 +735,6 @@ cudaError_t launch_mask_counts(const uint8_t* mask, int32_t m, int32_t* counts, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_unpermute(const float* zp, const int32_t* perm, int32_t m, float* z, cudaStream_t stream) {
-    k_unpermute<<<blocks_for(m, 256), 256, 0, stream>>>(zp, perm, m, z);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_permute_in(const float* src, const uint8_t* src_mask, const int32_t* perm, int32_t m,
                               int32_t m_pad, float* dst, uint8_t* dst_mask, cudaStream_t stream) {
     k_permute_in<<<blocks_for(m_pad, 256), 256, 0, stream>>>(src, src_mask, perm, m, m_pad, dst, dst_mask);
@@ -796,11 +783,6 @@ cudaError_t launch_row_absmax(const int64_t* t_off, const int64_t* col_len, cons
 cudaError_t launch_scales(const uint32_t* absmax_bits, int32_t n, int32_t n_pad, float qmax, float* scale,
                           float* inv_scale, cudaStream_t stream) {
     k_scales<<<blocks_for(n_pad, 256), 256, 0, stream>>>(absmax_bits, n, n_pad, qmax, scale, inv_scale);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_g_objective(const double* gpart, int32_t count, double* out, cudaStream_t stream) {
-    k_sum_doubles<<<1, 1024, 0, stream>>>(gpart, count, out);
     return cudaGetLastError();
 }
 

@@ -128,7 +128,6 @@ struct SolveParams {
 // Vectors of one plan.
 struct Vecs {
     float* x;        // kSets * n_pad
-    float* z;        // kSets * m_pad
     float* r;        // kSets * m_pad
     float* g;        // n_pad
     double* dpart;   // kMaxTrials * fwd_grid: per-CTA ||x_t - x||^2 partials
@@ -206,8 +205,10 @@ struct FwdArgs {
     const volatile int32_t* cancel;  // mapped host flag: nonzero asks the solve to stop
     const float* x_src;  // kFwdEval / kFwdPower: x (n_pad); NULL => accepted x; kFwdPowerNext: w
     float* v_dst;        // kFwdPowerNext: CTA 0 stores v = w / ||w|| here (n_pad)
-    float* z_dst;        // kFwdEval / kFwdPower; NULL => accepted set
-    float* r_dst;
+    float* z_dst;        // kFwdEval: the dose, or NULL (not stored; solves do not read it)
+    float* r_dst;        // kFwdEval / kFwdPower; NULL => accepted set
+    double* G_out;       // the last CTA adds the objective partials into it, or NULL (control 0)
+    int32_t z_caller;    // 1: z_dst is in the caller's voxel order (m entries), else permuted
     // the transposed pass that follows (segmented copies), for an L2 prefetch of its first rows
     // at the end of this pass; nx_tab NULL: none. nx_tab holds nx_per_cta (first entry, entries)
     // pairs per CTA (entries 0: nothing), one per warp w < nx_per_cta: the row that CTA
@@ -356,7 +357,6 @@ cudaError_t launch_tq_fill(int precision, const int64_t* t_off, const int32_t* t
                            const int64_t* col_len, int32_t n, int32_t H, const int64_t* seg, const float* inv_scale,
                            float* s_val, void* q_val, uint16_t* q_lo, cudaStream_t stream);
 cudaError_t launch_mask_counts(const uint8_t* mask, int32_t m, int32_t* counts, cudaStream_t stream);
-cudaError_t launch_unpermute(const float* zp, const int32_t* perm, int32_t m, float* z, cudaStream_t stream);
 cudaError_t launch_pad_copy(const float* src, int32_t n, int32_t n_pad, float* dst, cudaStream_t stream);
 cudaError_t launch_fill(float* dst, float v, int32_t count, cudaStream_t stream);
 // Keeps the stream busy for `ns` nanoseconds of device time (profiled host-driven solves: the
@@ -372,7 +372,6 @@ cudaError_t launch_row_absmax(const int64_t* t_off, const int64_t* col_len, cons
                               uint32_t* absmax_bits, cudaStream_t stream);
 cudaError_t launch_scales(const uint32_t* absmax_bits, int32_t n, int32_t n_pad, float qmax, float* scale,
                           float* inv_scale, cudaStream_t stream);
-cudaError_t launch_g_objective(const double* gpart, int32_t count, double* out, cudaStream_t stream);
 // The forward pass's L2 prefetch targets (FwdArgs::nx_tab): for t < count, the first entry of row
 // order[t] of the segmented beamlet-major copy and min(its entries, cap); (0, 0) for t >= n.
 cudaError_t launch_prefetch_table(const int32_t* order, const int64_t* seg, int32_t H, int32_t n, int32_t count,

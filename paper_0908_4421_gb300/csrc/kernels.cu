@@ -237,6 +237,23 @@ __device__ void control_step(int phase, DevState* st, const Vecs& v, const FwdUn
     }
 }
 
+// G of a stand-alone evaluation: the launch's objective partials added by its last CTA (fixed
+// order: per thread, the xor tree of each warp, then the warps), so no second kernel is needed.
+__device__ __forceinline__ void write_objective(const FwdUnits& U, double* G_out) {
+    __shared__ double part[32];
+    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5, nw = blockDim.x >> 5;
+    double t = 0.0;
+    for (int i = tid; i < U.n_obj; i += blockDim.x) t += __ldcg(U.obj + i);
+    if (wib * 32 < U.n_obj) t = warp_sum(t);  // (FP64 is scarce: idle warps skip it)
+    if (lane == 0) part[wib] = t;
+    __syncthreads();
+    if (tid == 0) {
+        double G = 0.0;
+        for (int k = 0; k < nw && k * 32 < U.n_obj; ++k) G += part[k];
+        *G_out = G;
+    }
+}
+
 // A slice's objective partials (one per trial, fixed shuffle order), then the group of
 // kGroupSlices consecutive slices it belongs to: the warp that completes the group (integer
 // arrival counter) adds the group's partials in slice order, so the controller only adds
@@ -292,7 +309,7 @@ struct LocalTables {
 // the last piece to arrive adds them in piece order; then, for complete rows, the penalty
 // epilogue writes z and r and the slice's objective partials.
 template <int KT, bool LOCAL>
-__device__ __forceinline__ void unit_epilogue(const FwdArgs& a, const Terms& T, int mode, float* const (&zq)[KT],
+__device__ __forceinline__ void unit_epilogue(const FwdArgs& a, const Terms& T, int mode, float* z,
                                               float* const (&rq)[KT], const UnitRec& R, int lane,
                                               const LocalTables& lt, float (&acc)[KT]) {
     const FwdUnits& U = a.u;
@@ -334,16 +351,13 @@ __device__ __forceinline__ void unit_epilogue(const FwdArgs& a, const Terms& T, 
         const uint32_t tg = a.vt ? a.vtm[p] : 0u;
         const int ro = a.r_index[p];
         if (mode == kFwdPower || mode == kFwdPowerNext) {
-            zq[0][p] = acc[0];
             rq[0][ro] = cdiag(bits, T, tg) * acc[0];
         } else {
             float rj[KT];
             penalty_multi<KT>(acc, bits, T, Fq, rj, tj, tg);
+            if (KT == 1 && z) z[a.z_caller ? ro : p] = acc[0];
 #pragma unroll
-            for (int q = 0; q < KT; ++q) {
-                zq[q][p] = acc[q];
-                rq[q][ro] = rj[q];
-            }
+            for (int q = 0; q < KT; ++q) rq[q][ro] = rj[q];
         }
     }
     if constexpr (LOCAL) {
@@ -641,16 +655,15 @@ __global__ void __launch_bounds__(kFwdThreads,
     }
 
     // Rows: work units taken dynamically, longest first.
-    float* zq[KT];
+    // the dose is stored only where a caller asks for it: nothing in a solve reads it
+    float* z = mode == kFwdEval ? a.z_dst : nullptr;
     float* rq[KT];
 #pragma unroll
     for (int q = 0; q < KT; ++q) {
         if (mode == kFwdTrial) {
             const int set = (cur + 1 + q) % kSets;
-            zq[q] = a.v.z + (size_t)set * a.m_pad;
             rq[q] = a.v.r + (size_t)set * a.m_pad;
         } else {
-            zq[q] = a.z_dst ? a.z_dst : a.v.z + (size_t)st->cur * a.m_pad;
             rq[q] = a.r_dst ? a.r_dst : a.v.r + (size_t)st->cur * a.m_pad;
         }
     }
@@ -670,7 +683,7 @@ __global__ void __launch_bounds__(kFwdThreads,
 #pragma unroll
             for (int q = 0; q < KT; ++q) acc[q] = 0.0f;
             slice_row_dot<F, KT>(a.val, a.col, R.off, R.g0, R.g1, lane, xs, acc);
-            unit_epilogue<KT, true>(a, T, mode, zq, rq, R, lane, lt, acc);
+            unit_epilogue<KT, true>(a, T, mode, z, rq, R, lane, lt, acc);
             u = __shfl_sync(0xffffffffu, u_next, 0);
         }
         __syncthreads();
@@ -698,7 +711,7 @@ __global__ void __launch_bounds__(kFwdThreads,
 #pragma unroll
             for (int q = 0; q < KT; ++q) acc[q] = 0.0f;
             slice_row_dot<F, KT>(a.val, a.col, R.off, R.g0, R.g1, lane, xs, acc);
-            unit_epilogue<KT, false>(a, T, mode, zq, rq, R, lane, lt, acc);
+            unit_epilogue<KT, false>(a, T, mode, z, rq, R, lane, lt, acc);
             u = __shfl_sync(0xffffffffu, u_next, 0);
         }
     }
@@ -718,6 +731,7 @@ __global__ void __launch_bounds__(kFwdThreads,
     __threadfence();
     if (!U.local) clear_group_counters(U);
     if (a.control) control_step<KT>(mode == kFwdTrial ? 1 : 0, st, a.v, U, a.n, gridDim.x, cs, cancel_req);
+    else if (a.G_out) write_objective(U, a.G_out);
     if (tid == 0) {
         *U.next_unit = 0;
         *U.ticket = 0;
@@ -1019,17 +1033,16 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_forward_tma(const FwdArgs a)
     } else if (wib - 1 < NC) {
         // ---- consumers ----
         const int c = wib - 1;
-        float* zq[KT];
+        // the dose is stored only where a caller asks for it: nothing in a solve reads it
+        float* z = mode == kFwdEval ? a.z_dst : nullptr;
         float* rq[KT];
 #pragma unroll
         for (int q = 0; q < KT; ++q) {
             if (mode == kFwdTrial) {
                 const int set = (cur + 1 + q) % kSets;
-                zq[q] = a.v.z + (size_t)set * a.m_pad;
-                rq[q] = a.v.r + (size_t)set * a.m_pad;
+                    rq[q] = a.v.r + (size_t)set * a.m_pad;
             } else {
-                zq[q] = a.z_dst ? a.z_dst : a.v.z + (size_t)st->cur * a.m_pad;
-                rq[q] = a.r_dst ? a.r_dst : a.v.r + (size_t)st->cur * a.m_pad;
+                    rq[q] = a.r_dst ? a.r_dst : a.v.r + (size_t)st->cur * a.m_pad;
             }
         }
         float acc[KT];
@@ -1067,16 +1080,13 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_forward_tma(const FwdArgs a)
                 const uint32_t tg = a.vt ? a.vtm[p] : 0u;
                 const int ro = a.r_index[p];
                 if (mode == kFwdPower) {
-                    zq[0][p] = acc[0];
                     rq[0][ro] = cdiag(bits, T, tg) * acc[0];
                 } else {
                     float rj[KT];
                     penalty_multi<KT>(acc, bits, T, Fq, rj, tj, tg);
+                    if (KT == 1 && z) z[a.z_caller ? ro : p] = acc[0];
 #pragma unroll
-                    for (int q = 0; q < KT; ++q) {
-                        zq[q][p] = acc[q];
-                        rq[q][ro] = rj[q];
-                    }
+                    for (int q = 0; q < KT; ++q) rq[q][ro] = rj[q];
                 }
             }
             publish_objective<KT>(U, mt.s, lane, Fq);
@@ -1092,6 +1102,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_forward_tma(const FwdArgs a)
     __threadfence();
     clear_group_counters(U);
     if (a.control) control_step<KT>(mode == kFwdTrial ? 1 : 0, st, a.v, U, a.n, gridDim.x, cs, cancel_req);
+    else if (a.G_out) write_objective(U, a.G_out);
     if (tid == 0) {
         *U.next_unit = 0;
         *U.ticket = 0;
