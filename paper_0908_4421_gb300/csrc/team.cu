@@ -36,6 +36,15 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned int* p) {
     return v;
 }
 
+// Adds to a word with release semantics: with the CTA barrier before it, every write of the CTA is visible
+// to the thread that acquires the sum.
+__device__ __forceinline__ void red_release_add(unsigned int* p, unsigned v) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// Polls before a waiting CTA yields between polls: most barriers fill within a few microseconds (64-plan
+// batch 35.6 ms polling without a pause, 36.0-36.2 ms with one from the first or the 65th poll on).
+constexpr unsigned kTeamBusySpins = 1u << 16;
+
 // Data another CTA of the team wrote during this launch comes from L2 (never a stale L1 line);
 // a one-CTA team reads its own writes through L1, which __syncthreads keeps coherent.
 template <class T>
@@ -50,8 +59,7 @@ __device__ bool team_barrier(const TeamPlan& P, unsigned k) {
     __syncthreads();
     if (P.team_size == 1) return true;
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(&P.sync[0], 1u);
+        red_release_add(&P.sync[0], 1u);
         const unsigned target = k * (unsigned)P.team_size;
         unsigned spins = 0;
         int good = 1;
@@ -60,20 +68,21 @@ __device__ bool team_barrier(const TeamPlan& P, unsigned k) {
                 good = 0;
                 break;
             }
-            __nanosleep(64);
+            if (spins > kTeamBusySpins) __nanosleep(64);
         }
-        __threadfence();
         ok = good;
     }
     __syncthreads();
     return ok != 0;
 }
 
-// Fixed-order CTA reduction of NQ double-float values per thread into out[q] (thread-strided
-// order, then a shuffle tree per warp, then the warps in index order; one conversion to double).
+// Fixed-order CTA reduction of NQ double-float values per thread, in two steps with a CTA barrier
+// between them: a shuffle tree per warp into red[warp][q], then for each value the xor tree over the
+// 16 warps' sums, 16 threads a value starting at thread `first` (one thread adding the 16 in turn was
+// a long dependent chain, twice a pass); one conversion to double.
+using CtaRed = Df[kTW][kMaxTrials];
 template <int NQ>
-__device__ __forceinline__ void cta_sum(Df (&v)[NQ], double* out) {
-    __shared__ Df red[kTW][kMaxTrials];
+__device__ __forceinline__ void cta_sum_warps(Df (&v)[NQ], CtaRed& red) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     if constexpr (NQ == 1) {
         const Df t = warp_sum(v[0]);
@@ -82,19 +91,37 @@ __device__ __forceinline__ void cta_sum(Df (&v)[NQ], double* out) {
         const Df t = warp_sum_multi<NQ>(v, lane);
         if ((lane & (32 / NQ - 1)) == 0) red[wib][warp_sum_multi_q<NQ>(lane)] = t;
     }
-    __syncthreads();
-    if (threadIdx.x < NQ) {
-        Df t = red[0][threadIdx.x];
-        for (int w = 1; w < kTW; ++w) t = df_add(t, red[w][threadIdx.x]);
-        out[threadIdx.x] = df_to_double(t);
+}
+template <int NQ>
+__device__ __forceinline__ void cta_sum_final(const CtaRed& red, int first, double* out) {
+    static_assert(kTW == 16, "16 threads a value");
+    constexpr int kThreads = (16 * NQ + 31) / 32 * 32;  // whole warps
+    const int t = (int)threadIdx.x - first;
+    if (t < 0 || t >= kThreads) return;
+    const int q = t >> 4, w = t & 15;
+    Df v = q < NQ ? red[w][q] : Df{0.0f, 0.0f};
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+        Df u;
+        u.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
+        u.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
+        v = df_add(v, u);
     }
+    if (q < NQ && w == 0) out[q] = df_to_double(v);
+}
+template <int NQ>
+__device__ __forceinline__ void cta_sum(Df (&v)[NQ], CtaRed& red, double* out) {
+    cta_sum_warps<NQ>(v, red);
+    __syncthreads();
+    cta_sum_final<NQ>(red, 0, out);
     __syncthreads();
 }
 
 // The busy slices' part of G for every evaluated step size: their partials (double-float pairs,
-// stored by unit index) added in unit order.
+// stored by unit index) added in unit order
+// (their sums per warp, into red).
 template <int NQ>
-__device__ __forceinline__ void sum_objective(const TeamPlan& P, const double* objb, int nq, double* out) {
+__device__ __forceinline__ void sum_objective(const TeamPlan& P, const double* objb, int nq, CtaRed& red) {
     const bool multi = P.team_size > 1;
     const float2* ob = reinterpret_cast<const float2*>(objb);
     Df v[NQ];
@@ -108,12 +135,12 @@ __device__ __forceinline__ void sum_objective(const TeamPlan& P, const double* o
                 v[q] = df_add(v[q], Df{w.x, w.y});
             }
     }
-    cta_sum<NQ>(v, out);
+    cta_sum_warps<NQ>(v, red);
 }
 
 // The slices without entries: their dose is 0 at every x, so their part of G is one constant,
 // summed once per solve from the partials the evaluation pass left (idle list order).
-__device__ __forceinline__ void sum_idle(const TeamPlan& P, double* out) {
+__device__ __forceinline__ void sum_idle(const TeamPlan& P, CtaRed& red, double* out) {
     const bool multi = P.team_size > 1;
     const float2* ob = reinterpret_cast<const float2*>(P.obj) + (size_t)2 * kMaxTrials * P.n_busy;
     Df v[1] = {Df{0.0f, 0.0f}};
@@ -121,7 +148,7 @@ __device__ __forceinline__ void sum_idle(const TeamPlan& P, double* out) {
         const float2 w = ld_team(ob + u, multi);
         v[0] = df_add(v[0], Df{w.x, w.y});
     }
-    cta_sum<1>(v, out);
+    cta_sum<1>(v, red, out);
 }
 
 // The penalty epilogue of one slice (Eq. (1)): r of its 32 voxels for the evaluated step sizes
@@ -612,6 +639,7 @@ struct TeamShared {
     Terms T;
     double sums[kMaxTrials];
     double d2[kMaxTrials];
+    CtaRed red, red_d;      // warp sums of the objective and of ||x_t - x||^2
     float ginf[kTW];
     int64_t sb[kTW][17];
     TeamCtl c;
@@ -673,9 +701,12 @@ __device__ __noinline__ int2 team_solve(int rank, float* smem, TeamShared& sh, b
     const size_t obj_buf = (size_t)kMaxTrials * P.n_busy;
     team_forward<F, 1>(P, sh.T, xs, 0, true, gw, W, P.obj);  // pass 0: buffer 0
     bool fail = !team_barrier(P, ++bar);
-    sum_idle(P, sh.sums);
+    sum_idle(P, sh.red, sh.sums);
     const double G_idle = sh.sums[0];  // every CTA of the team holds the same
-    sum_objective<1>(P, P.obj, 1, sh.sums);
+    sum_objective<1>(P, P.obj, 1, sh.red);
+    __syncthreads();
+    cta_sum_final<1>(sh.red, 0, sh.sums);
+    __syncthreads();
     double G = sh.sums[0] + G_idle;
     const double G0 = G;
     int status = bad_x ? (int)IMRT_EINVAL : 0, stop = 0;
@@ -698,9 +729,11 @@ __device__ __noinline__ int2 team_solve(int rank, float* smem, TeamShared& sh, b
             gs[i] = g;
             gm = fmaxf(gm, fabsf(g));
         }
+        if (!g1_done) {  // ||g(x_1)||_inf
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) gm = fmaxf(gm, __shfl_xor_sync(0xffffffffu, gm, o));
-        if (lane == 0) sh.ginf[wib] = gm;
+            for (int o = 16; o > 0; o >>= 1) gm = fmaxf(gm, __shfl_xor_sync(0xffffffffu, gm, o));
+            if (lane == 0) sh.ginf[wib] = gm;
+        }
         __syncthreads();
         if (!g1_done) {
             float t = 0.0f;
@@ -717,6 +750,21 @@ __device__ __noinline__ int2 team_solve(int rank, float* smem, TeamShared& sh, b
     // arithmetic would otherwise run 512 times over on a part with a small FP64 rate) and every
     // thread reads the outcome after a barrier.
     TeamCtl& c = sh.c;
+    // (one thread) the step sizes of the next trial pass; step 2 of an iteration
+    auto set_steps = [&]() {
+        double l = c.lam;
+#pragma unroll
+        for (int q = 0; q < KT; ++q) {
+            sh.lam[q] = (float)l;
+            if (q + 1 < KT) l = l * sp.inv_alpha;
+        }
+    };
+    auto start_iteration = [&]() {
+        c.lam = sp.lambda0;
+        c.eol = sp.eps_over_lambda0;
+        c.bt = 0;
+        set_steps();
+    };
     if (tid == 0) {
         c.G = G;
         c.dG = 0.0;
@@ -726,6 +774,7 @@ __device__ __noinline__ int2 team_solve(int rank, float* smem, TeamShared& sh, b
         c.cur = 0;
         c.iter = 0;
         c.total_bt = 0;
+        start_iteration();
     }
     __syncthreads();
     while (status == 0 && stop == 0) {
@@ -733,22 +782,9 @@ __device__ __noinline__ int2 team_solve(int rank, float* smem, TeamShared& sh, b
             status = IMRT_ECUDA;
             break;
         }
-        if (tid == 0) {
-            c.lam = sp.lambda0;
-            c.eol = sp.eps_over_lambda0;
-            c.bt = 0;
-        }
         while (status == 0 && stop == 0) {
-            // trial points of the KT step sizes lam, lam / alpha, ... and their ||x_t - x||^2
-            if (tid == 0) {
-                double l = c.lam;
-#pragma unroll
-                for (int q = 0; q < KT; ++q) {
-                    sh.lam[q] = (float)l;
-                    l = l * sp.inv_alpha;
-                }
-            }
-            __syncthreads();
+            // trial points of the KT step sizes lam, lam / alpha, ... (sh.lam, set with the decision
+            // before) and their ||x_t - x||^2
             float lamf[KT];
 #pragma unroll
             for (int q = 0; q < KT; ++q) lamf[q] = sh.lam[q];
@@ -774,7 +810,8 @@ __device__ __noinline__ int2 team_solve(int rank, float* smem, TeamShared& sh, b
                     d2[q] = df_add(d2[q], Df{sq.hi, fmaf(2.0f * dh, dl, sq.lo)});
                 }
             }
-            cta_sum<KT>(d2, sh.d2);  // also makes xs visible to every warp
+            cta_sum_warps<KT>(d2, sh.red_d);
+            __syncthreads();  // xs is visible to every warp
             double* objb = P.obj + (size_t)(passes & 1) * obj_buf;
             team_forward_ring<F, KT>(P, sh.T, xs, sh.lam, cur, gw, W, objb, ring);
             ++passes;
@@ -794,7 +831,11 @@ __device__ __noinline__ int2 team_solve(int rank, float* smem, TeamShared& sh, b
             }
             // the stop request's load is issued before the sums, which hide its latency
             const unsigned req = tid == 0 ? ld_team(&P.sync[1 + (bar & 1)], multi) : 0u;
-            sum_objective<KT>(P, objb, KT, sh.sums);
+            sum_objective<KT>(P, objb, KT, sh.red);
+            __syncthreads();
+            cta_sum_final<KT>(sh.red, 0, sh.sums);
+            cta_sum_final<KT>(sh.red_d, kTeamThreads / 2, sh.d2);
+            __syncthreads();
             if (tid == 0) {
                 // Eq. (5) for the step sizes in order (the sequential Armijo decisions)
                 int accepted = -1;
@@ -837,11 +878,13 @@ __device__ __noinline__ int2 team_solve(int rank, float* smem, TeamShared& sh, b
                     else if (c.dG < sp.delta * Gt) c.stop = IMRT_STOP_REL;  // step 5: |dG| / G < delta
                     else if (c.iter >= sp.max_iter) c.stop = IMRT_STOP_MAXITER;
                     if (c.stop == 0 && req) c.status = req == 1 ? IMRT_ECANCELLED : IMRT_ETIMEOUT;
+                    start_iteration();
                 } else {
                     if (c.status == 0 && c.stop == 0) {
                         if (c.bt + KT - 1 >= sp.max_bt) c.status = IMRT_ELINESEARCH;
                         else {
                             c.bt += KT;
+                            set_steps();
                             if (req) c.status = req == 1 ? IMRT_ECANCELLED : IMRT_ETIMEOUT;
                         }
                     }
