@@ -971,27 +971,27 @@ imrt_status plan_build(imrt_plan* p, const imrt_csr* D, const uint8_t* structure
     CK(cudaMemcpyAsync(hlen.data(), col_len, sizeof(int64_t) * n, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     // Plans with at most 16 segments of 65536 voxels keep segmented beamlet-major copies (16-bit
-    // voxel offsets: 6 bytes per FP32 entry); the int32-index copy is then only the source
-    // of the segmented ones and is freed with the build's temporaries.
+    // voxel offsets: 6 bytes per FP32 entry), cut from (value, voxel) pairs that are freed with the
+    // build's temporaries; others keep the int32-index copy.
     const int H = (int)((p->m_pad + 65535) / 65536);
     const bool segmented = H <= kMaxSegments;
     if (!segmented && p->opt.precision != IMRT_FP32)
         return set_error("reduced precision supports at most 1048576 voxels"), IMRT_EUNSUPPORTED;
-    Temp tval_src, trow_src;
+    Temp tpair;
+    uint2* pair = nullptr;
     if (segmented) {
-        TRY(talloc(tval_src, &p->t_val, p->t_entries + 4));
-        TRY(talloc(trow_src, &p->t_row, p->t_entries + 4));
+        TRY(talloc(tpair, &pair, p->t_entries + 4));
     } else {
         TRY(dalloc(p, &p->t_val, p->t_entries + 4));
         TRY(dalloc(p, &p->t_row, p->t_entries + 4));
     }
-    CK(launch_transpose_fill(row_ptr, col, val, p->m, n, chunk_rows, counts, col_len, p->t_off, p->t_val,
-                             p->t_row, s));
+    CK(launch_transpose_fill(row_ptr, col, val, p->m, n, chunk_rows, counts, col_len, p->t_off, pair, p->t_val, p->t_row,
+                             s));
     if (p->opt.precision != IMRT_FP32) {  // (segmented) per-beamlet scales, then the reduced voxel-major copy
         Temp tabs;
         uint32_t* absmax;
         TRY(talloc(tabs, &absmax, n));
-        CK(launch_row_absmax(p->t_off, col_len, p->t_val, n, absmax, s));
+        CK(launch_row_absmax(p->t_off, col_len, pair, n, absmax, s));
         TRY(dalloc(p, &p->scale, p->n_pad));
         TRY(dalloc(p, &p->inv_scale, p->n_pad));
         const float qmax = p->opt.precision == IMRT_FP8E4M3 ? 448.0f : 1.0f;
@@ -1004,7 +1004,7 @@ imrt_status plan_build(imrt_plan* p, const imrt_csr* D, const uint8_t* structure
         int64_t* seg_len;
         TRY(talloc(tsl, &seg_len, (size_t)n * H));
         TRY(dalloc(p, &p->t_seg, (size_t)n * H + 1));
-        CK(launch_tq_count(p->t_off, p->t_row, col_len, n, H, seg_len, s));
+        CK(launch_tq_count(p->t_off, pair, col_len, n, H, seg_len, s));
         CK(launch_scan_i64(seg_len, p->t_seg, (int64_t)n * H, s));
         CK(cudaMemcpyAsync(&p->tq_entries, p->t_seg + (size_t)n * H, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
@@ -1012,12 +1012,11 @@ imrt_status plan_build(imrt_plan* p, const imrt_csr* D, const uint8_t* structure
         TRY(dalloc(p, &p->t_vals, (size_t)p->tq_entries + 16));
         if (p->opt.precision != IMRT_FP32)
             TRY(dalloc_bytes(p, &p->t_valq, (size_t)p->tq_entries * elem_bytes(p->opt.precision) + 64));
-        CK(launch_tq_fill(p->opt.precision, p->t_off, p->t_row, p->t_val, col_len, n, H, p->t_seg, p->inv_scale,
+        CK(launch_tq_fill(p->opt.precision, p->t_off, pair, col_len, n, H, p->t_seg, p->inv_scale,
                           p->t_vals, p->t_valq, p->t_lo, s));
         CK(cudaStreamSynchronize(s));
     }
     TRY(make_bwd_schedule(p, hlen));
-    if (segmented) p->t_val = nullptr, p->t_row = nullptr;  // freed with the temporaries below
     // --- structures and term coefficients (Eq. (1): c = w / |V_s|) ----------
     Temp tcnt;
     int32_t* scount;

@@ -287,13 +287,31 @@ __global__ void __launch_bounds__(32 * kScanParts) k_t_colscan(int32_t* __restri
     }
 }
 
+// Where the scatter puts an entry of the beamlet-major rows: (value, voxel) pairs of 8 bytes when the rows are
+// only the source of the segmented copies, else the plan's two arrays. The scatter is bound by its
+// stores, each lane's in a sector of its own: one per entry instead of two (61M entries: 1.88 -> 1.07 ms).
+struct TDest {
+    uint2* pair;
+    float* val;
+    int32_t* row;
+};
+template <bool PAIR>
+__device__ __forceinline__ void store_t(const TDest& o, int64_t k, float v, int32_t row) {
+    if constexpr (PAIR) {
+        o.pair[k] = make_uint2(__float_as_uint(v), (uint32_t)row);
+    } else {
+        o.val[k] = v;
+        o.row[k] = row;
+    }
+}
+
 // Pass 3: scatter. Rows of a chunk are visited in order, so each beamlet row
 // receives voxels in ascending (caller) index; within one voxel row the
 // columns are distinct, so the per-beamlet cursors need no atomics.
+template <bool PAIR>
 __global__ void k_t_scatter(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                             const float* __restrict__ val, int32_t m, int32_t n, int32_t chunk_rows,
-                            const int32_t* __restrict__ counts, const int64_t* __restrict__ t_off,
-                            float* __restrict__ t_val, int32_t* __restrict__ t_row) {
+                            const int32_t* __restrict__ counts, const int64_t* __restrict__ t_off, TDest out) {
     extern __shared__ int32_t cursor[];
     for (int c = threadIdx.x; c < n; c += blockDim.x) cursor[c] = counts[(size_t)blockIdx.x * n + c];
     __syncthreads();
@@ -305,9 +323,7 @@ __global__ void k_t_scatter(const int64_t* __restrict__ row_ptr, const int32_t* 
             const int c = col[k];
             const int pos = cursor[c];
             cursor[c] = pos + 1;
-            const int64_t dst = t_off[c] + pos;
-            t_val[dst] = val[k];
-            t_row[dst] = j;
+            store_t<PAIR>(out, t_off[c] + pos, val[k], j);
         }
         __syncthreads();
     }
@@ -322,10 +338,10 @@ __global__ void k_t_scatter(const int64_t* __restrict__ row_ptr, const int32_t* 
 // in flight per lane). (Splitting the launch into beamlet ranges whose writes stay in L2 was
 // measured slower: every range re-reads the column indices.)
 constexpr int kTBlockRows = 32;
+template <bool PAIR>
 __global__ void k_t_scatter_blocks(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                                    const float* __restrict__ val, int32_t m, int32_t n, int32_t chunk_rows,
-                                   const int32_t* __restrict__ counts, const int64_t* __restrict__ t_off,
-                                   float* __restrict__ t_val, int32_t* __restrict__ t_row) {
+                                   const int32_t* __restrict__ counts, const int64_t* __restrict__ t_off, TDest out) {
     extern __shared__ int32_t cursor[];                      // n: position within the beamlet row
     uint32_t* mask = reinterpret_cast<uint32_t*>(cursor + n);  // n: rows of the block holding the beamlet
     __shared__ int64_t rp[kTBlockRows + 1];
@@ -370,8 +386,7 @@ __global__ void k_t_scatter_blocks(const int64_t* __restrict__ row_ptr, const in
                     const int c = cc[u];
                     if (c < 0) continue;
                     const int64_t dst = __ldg(t_off + c) + cursor[c] + __popc(mask[c] & below);
-                    t_val[dst] = vv[u];
-                    t_row[dst] = jb + r;
+                    store_t<PAIR>(out, dst, vv[u], jb + r);
                 }
             }
         }
@@ -399,23 +414,23 @@ __global__ void k_t_pad(const int64_t* __restrict__ col_len, const int64_t* __re
 // Reduced-precision beamlet-major copy with 16-bit voxel indices: row i is cut into
 // segments h = voxel >> 16 (the row is sorted, so each segment is one contiguous run,
 // found by binary search); each segment is padded to a multiple of 8 entries.
-__device__ __forceinline__ int64_t lower_bound_row(const int32_t* __restrict__ row, int64_t a, int64_t b, int32_t v) {
+__device__ __forceinline__ int64_t lower_bound_row(const uint2* __restrict__ pair, int64_t a, int64_t b, int32_t v) {
     while (a < b) {
         const int64_t mid = (a + b) >> 1;
-        if (row[mid] < v) a = mid + 1;
+        if ((int32_t)pair[mid].y < v) a = mid + 1;
         else b = mid;
     }
     return a;
 }
 
-__global__ void k_tq_count(const int64_t* __restrict__ t_off, const int32_t* __restrict__ t_row,
+__global__ void k_tq_count(const int64_t* __restrict__ t_off, const uint2* __restrict__ pair,
                            const int64_t* __restrict__ col_len, int32_t n, int32_t H, int64_t* __restrict__ seg_len) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int64_t a = t_off[i], b = a + col_len[i];
     int64_t prev = a;
     for (int h = 0; h < H; ++h) {
-        const int64_t e = h + 1 < H ? lower_bound_row(t_row, a, b, (h + 1) << 16) : b;
+        const int64_t e = h + 1 < H ? lower_bound_row(pair, a, b, (h + 1) << 16) : b;
         const int64_t len = e - prev;
         seg_len[(int64_t)i * H + h] = (len + 7) & ~(int64_t)7;
         prev = e;
@@ -428,8 +443,8 @@ __global__ void k_tq_count(const int64_t* __restrict__ t_off, const int32_t* __r
 // row and its writes whole 16-byte words. 61M entries, FP32 + FP16: 0.17 ms (0.14 ms at the copy rate);
 // one thread an entry, with a division by sg for its place, and a launch a copy took 0.40 + 0.34 ms.
 template <int PREC>
-__global__ void __launch_bounds__(256) k_tq_fill(const int64_t* __restrict__ t_off, const int32_t* __restrict__ t_row,
-                                                 const float* __restrict__ t_val, const int64_t* __restrict__ col_len,
+__global__ void __launch_bounds__(256) k_tq_fill(const int64_t* __restrict__ t_off, const uint2* __restrict__ pair,
+                                                 const int64_t* __restrict__ col_len,
                                                  int32_t n, int32_t H, const int64_t* __restrict__ seg,
                                                  const float* __restrict__ inv_scale, float* __restrict__ s_val,
                                                  void* q_val, uint16_t* __restrict__ q_lo) {
@@ -440,7 +455,7 @@ __global__ void __launch_bounds__(256) k_tq_fill(const int64_t* __restrict__ t_o
     if (threadIdx.x <= H) {
         const int h = threadIdx.x;
         sb[h] = seg[(int64_t)i * H + h];
-        src[h] = h == 0 ? a : h == H ? b : lower_bound_row(t_row, a, b, h << 16);
+        src[h] = h == 0 ? a : h == H ? b : lower_bound_row(pair, a, b, h << 16);
     }
     __syncthreads();
     const int64_t r0 = sb[0];
@@ -460,8 +475,9 @@ __global__ void __launch_bounds__(256) k_tq_fill(const int64_t* __restrict__ t_o
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
             const bool in = f + t * sg < src[h + 1];
-            v[t] = in ? __ldg(t_val + f + t * sg) : 0.0f;
-            lo[t] = in ? (uint32_t)__ldg(t_row + f + t * sg) & 0xffffu : 0u;
+            const uint2 w = in ? __ldg(pair + f + t * sg) : make_uint2(0u, 0u);
+            v[t] = __uint_as_float(w.x);
+            lo[t] = w.y & 0xffffu;
         }
         float4* sv = reinterpret_cast<float4*>(s_val + e);
         sv[0] = make_float4(v[0], v[1], v[2], v[3]);
@@ -544,10 +560,10 @@ __global__ void __launch_bounds__(256) k_sum_masked_part(const float* __restrict
     if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-// max |D_ij| of each beamlet, one CTA a row of the beamlet-major copy (coalesced: 43 us for
-// 61M entries, 36 at the copy rate; one thread a voxel row with an atomic maximum per entry took 3.1 ms).
+// max |D_ij| of each beamlet, one CTA a row of the beamlet-major pairs (coalesced: 73 us for
+// 61M entries of 8 bytes at the copy rate; one thread a voxel row with an atomic maximum per entry took 3.1 ms).
 __global__ void __launch_bounds__(256) k_row_absmax(const int64_t* __restrict__ t_off, const int64_t* __restrict__ col_len,
-                                                    const float* __restrict__ t_val, uint32_t* __restrict__ absmax_bits) {
+                                                    const uint2* __restrict__ pair, uint32_t* __restrict__ absmax_bits) {
     __shared__ uint32_t sh[8];
     const int i = blockIdx.x;
     const int64_t a = t_off[i], b = a + col_len[i];
@@ -556,7 +572,7 @@ __global__ void __launch_bounds__(256) k_row_absmax(const int64_t* __restrict__ 
     for (int64_t k = a + threadIdx.x; k < b; k += kU * 256) {
 #pragma unroll
         for (int u = 0; u < kU; ++u)
-            most = max(most, k + u * 256 < b ? __float_as_uint(fabsf(__ldg(t_val + k + u * 256))) : 0u);
+            most = max(most, k + u * 256 < b ? __ldg(pair + k + u * 256).x & 0x7fffffffu : 0u);  // |D_ij|
     }
     most = __reduce_max_sync(0xffffffffu, most);
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = most;
@@ -675,7 +691,9 @@ cudaError_t launch_transpose_plan(const int64_t* row_ptr, const int32_t* col, in
 
 cudaError_t launch_transpose_fill(const int64_t* row_ptr, const int32_t* col, const float* val, int32_t m,
                                   int32_t n, int32_t chunk_rows, const int32_t* counts, const int64_t* col_len,
-                                  const int64_t* t_off, float* t_val, int32_t* t_row, cudaStream_t stream) {
+                                  const int64_t* t_off, uint2* pair, float* t_val, int32_t* t_row,
+                                  cudaStream_t stream) {
+    const TDest out{pair, t_val, t_row};
     const int n_chunks = (m + chunk_rows - 1) / chunk_rows;
     int dev = 0, max_smem = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -684,44 +702,45 @@ cudaError_t launch_transpose_fill(const int64_t* row_ptr, const int32_t* col, co
     // the row-block scatter keeps a cursor and a mask per beamlet in shared memory; beyond that
     // room, the row-by-row scatter (a cursor per beamlet) gives the same copy
     const size_t smem2 = (size_t)n * 2 * sizeof(int32_t);
-    if (smem2 + 1024 <= (size_t)max_smem) {
-        if (smem2 > 48 * 1024 && (e = set_max_dynamic_smem(k_t_scatter_blocks)) != cudaSuccess) return e;
-        k_t_scatter_blocks<<<n_chunks, 256, smem2, stream>>>(row_ptr, col, val, m, n, chunk_rows, counts, t_off,
-                                                            t_val, t_row);
-    } else {
-        const size_t smem = (size_t)n * sizeof(int32_t);
-        if (smem > 48 * 1024 && (e = set_max_dynamic_smem(k_t_scatter)) != cudaSuccess) return e;
-        k_t_scatter<<<n_chunks, 256, smem, stream>>>(row_ptr, col, val, m, n, chunk_rows, counts, t_off, t_val,
-                                                     t_row);
-    }
+    const bool blocks = smem2 + 1024 <= (size_t)max_smem;
+    const size_t smem = blocks ? smem2 : (size_t)n * sizeof(int32_t);
+    auto launch = [&](auto kernel) {
+        cudaError_t r = smem > 48 * 1024 ? set_max_dynamic_smem(kernel) : cudaSuccess;
+        if (r != cudaSuccess) return r;
+        kernel<<<n_chunks, 256, smem, stream>>>(row_ptr, col, val, m, n, chunk_rows, counts, t_off, out);
+        return cudaGetLastError();
+    };
+    if (pair) return blocks ? launch(k_t_scatter_blocks<true>) : launch(k_t_scatter<true>);
+    e = blocks ? launch(k_t_scatter_blocks<false>) : launch(k_t_scatter<false>);
+    if (e != cudaSuccess) return e;
     k_t_pad<<<blocks_for(n, 256), 256, 0, stream>>>(col_len, t_off, n, t_val, t_row);
     return cudaGetLastError();
 }
 
-cudaError_t launch_tq_count(const int64_t* t_off, const int32_t* t_row, const int64_t* col_len, int32_t n, int32_t H,
+cudaError_t launch_tq_count(const int64_t* t_off, const uint2* pair, const int64_t* col_len, int32_t n, int32_t H,
                             int64_t* seg_len, cudaStream_t stream) {
-    k_tq_count<<<blocks_for(n, 128), 128, 0, stream>>>(t_off, t_row, col_len, n, H, seg_len);
+    k_tq_count<<<blocks_for(n, 128), 128, 0, stream>>>(t_off, pair, col_len, n, H, seg_len);
     return cudaGetLastError();
 }
 
-cudaError_t launch_tq_fill(int precision, const int64_t* t_off, const int32_t* t_row, const float* t_val,
-                           const int64_t* col_len, int32_t n, int32_t H, const int64_t* seg, const float* inv_scale,
+cudaError_t launch_tq_fill(int precision, const int64_t* t_off, const uint2* pair, const int64_t* col_len,
+                           int32_t n, int32_t H, const int64_t* seg, const float* inv_scale,
                            float* s_val, void* q_val, uint16_t* q_lo, cudaStream_t stream) {
     switch (precision) {
         case IMRT_FP32:
-            k_tq_fill<IMRT_FP32><<<n, 256, 0, stream>>>(t_off, t_row, t_val, col_len, n, H, seg, inv_scale, s_val, q_val,
+            k_tq_fill<IMRT_FP32><<<n, 256, 0, stream>>>(t_off, pair, col_len, n, H, seg, inv_scale, s_val, q_val,
                                                         q_lo);
             break;
         case IMRT_FP16:
-            k_tq_fill<IMRT_FP16><<<n, 256, 0, stream>>>(t_off, t_row, t_val, col_len, n, H, seg, inv_scale, s_val, q_val,
+            k_tq_fill<IMRT_FP16><<<n, 256, 0, stream>>>(t_off, pair, col_len, n, H, seg, inv_scale, s_val, q_val,
                                                         q_lo);
             break;
         case IMRT_BF16:
-            k_tq_fill<IMRT_BF16><<<n, 256, 0, stream>>>(t_off, t_row, t_val, col_len, n, H, seg, inv_scale, s_val, q_val,
+            k_tq_fill<IMRT_BF16><<<n, 256, 0, stream>>>(t_off, pair, col_len, n, H, seg, inv_scale, s_val, q_val,
                                                         q_lo);
             break;
         case IMRT_FP8E4M3:
-            k_tq_fill<IMRT_FP8E4M3><<<n, 256, 0, stream>>>(t_off, t_row, t_val, col_len, n, H, seg, inv_scale, s_val,
+            k_tq_fill<IMRT_FP8E4M3><<<n, 256, 0, stream>>>(t_off, pair, col_len, n, H, seg, inv_scale, s_val,
                                                            q_val, q_lo);
             break;
         default:
@@ -774,9 +793,9 @@ cudaError_t launch_sum_masked(const float* z, const uint8_t* mask, int32_t bit, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_row_absmax(const int64_t* t_off, const int64_t* col_len, const float* t_val, int32_t n,
+cudaError_t launch_row_absmax(const int64_t* t_off, const int64_t* col_len, const uint2* pair, int32_t n,
                               uint32_t* absmax_bits, cudaStream_t stream) {
-    k_row_absmax<<<n, 256, 0, stream>>>(t_off, col_len, t_val, absmax_bits);
+    k_row_absmax<<<n, 256, 0, stream>>>(t_off, col_len, pair, absmax_bits);
     return cudaGetLastError();
 }
 

@@ -346,15 +346,18 @@ cudaError_t launch_sell_fill(int fmt, const int64_t* row_ptr, const int32_t* col
 cudaError_t launch_transpose_plan(const int64_t* row_ptr, const int32_t* col, int32_t m, int32_t n,
                                   int32_t chunk_rows, int32_t* counts, int64_t* col_len, int64_t* padded,
                                   int64_t* t_off, cudaStream_t stream);
+// The beamlet-major rows, sorted by voxel: into (value, voxel) pairs if `pair` is given (the source of the
+// segmented copies), else into t_val / t_row with each row's padding.
 cudaError_t launch_transpose_fill(const int64_t* row_ptr, const int32_t* col, const float* val, int32_t m,
                                   int32_t n, int32_t chunk_rows, const int32_t* counts, const int64_t* col_len,
-                                  const int64_t* t_off, float* t_val, int32_t* t_row, cudaStream_t stream);
-cudaError_t launch_tq_count(const int64_t* t_off, const int32_t* t_row, const int64_t* col_len, int32_t n, int32_t H,
+                                  const int64_t* t_off, uint2* pair, float* t_val, int32_t* t_row,
+                                  cudaStream_t stream);
+cudaError_t launch_tq_count(const int64_t* t_off, const uint2* pair, const int64_t* col_len, int32_t n, int32_t H,
                             int64_t* seg_len, cudaStream_t stream);
 // The FP32 segmented copy (s_val, q_lo) and, for a reduced precision, its scaled values in the same places
 // (q_val; NULL with IMRT_FP32).
-cudaError_t launch_tq_fill(int precision, const int64_t* t_off, const int32_t* t_row, const float* t_val,
-                           const int64_t* col_len, int32_t n, int32_t H, const int64_t* seg, const float* inv_scale,
+cudaError_t launch_tq_fill(int precision, const int64_t* t_off, const uint2* pair, const int64_t* col_len,
+                           int32_t n, int32_t H, const int64_t* seg, const float* inv_scale,
                            float* s_val, void* q_val, uint16_t* q_lo, cudaStream_t stream);
 cudaError_t launch_mask_counts(const uint8_t* mask, int32_t m, int32_t* counts, cudaStream_t stream);
 cudaError_t launch_pad_copy(const float* src, int32_t n, int32_t n_pad, float* dst, cudaStream_t stream);
@@ -368,7 +371,7 @@ cudaError_t launch_sum_masked(const float* z, const uint8_t* mask, int32_t bit, 
 cudaError_t launch_permute_in(const float* src, const uint8_t* src_mask, const int32_t* perm, int32_t m,
                               int32_t m_pad, float* dst, uint8_t* dst_mask, cudaStream_t stream);
 // absmax_bits[i] = bits of max |D_ij| over row i of the beamlet-major copy (i < n).
-cudaError_t launch_row_absmax(const int64_t* t_off, const int64_t* col_len, const float* t_val, int32_t n,
+cudaError_t launch_row_absmax(const int64_t* t_off, const int64_t* col_len, const uint2* pair, int32_t n,
                               uint32_t* absmax_bits, cudaStream_t stream);
 cudaError_t launch_scales(const uint32_t* absmax_bits, int32_t n, int32_t n_pad, float qmax, float* scale,
                           float* inv_scale, cudaStream_t stream);
