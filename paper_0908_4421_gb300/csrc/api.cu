@@ -112,6 +112,7 @@ struct FwdShape {
     size_t smem = 0;
     size_t smem1 = 0;
     FwdUnits units{};
+    bool finished = false;      // finish_shape has run
     int64_t* pf_tab = nullptr;  // warp streaming: the L2 prefetch targets (FwdArgs::nx_tab), or none
     int pf_per_cta = 0;
 };
@@ -375,6 +376,19 @@ imrt_status validate_options(const imrt_options* o) {
 #define IMRT_FWD_PIECES 4  // pieces of a warp's share that bound a forward work unit
 #endif
 
+// Indices 0 .. count - 1 by class (ascending), cost (descending, below 2^40), index: sorted as packed keys, which
+// is several times faster than a stable sort through the arrays they come from.
+template <class C, class K>
+std::vector<int32_t> order_by(int count, C&& cls, K&& cost) {
+    std::vector<std::pair<uint64_t, int32_t>> key(count);
+    for (int i = 0; i < count; ++i)
+        key[i] = {((uint64_t)cls(i) << 40) | ((((uint64_t)1 << 40) - 1) - (uint64_t)cost(i)), i};
+    std::sort(key.begin(), key.end());
+    std::vector<int32_t> order(count);
+    for (int i = 0; i < count; ++i) order[i] = key[i].second;
+    return order;
+}
+
 imrt_status make_shape(imrt_plan* p, const SellCopy& c, int k_trials, int variant, FwdShape* out) {
     int max_smem = 0;
     CK(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
@@ -498,10 +512,8 @@ imrt_status make_shape(imrt_plan* p, const SellCopy& c, int k_trials, int varian
     if (local) {
         // CTA-local schedule: whole slices dealt to CTAs, longest first, each to the least-loaded
         // CTA (ties: the lower index); every CTA's units longest first
-        std::vector<int32_t> sorder(p->n_slices);
-        for (int s = 0; s < p->n_slices; ++s) sorder[s] = s;
-        std::stable_sort(sorder.begin(), sorder.end(),
-                         [&](int x, int y) { return c.host_cost[x] > c.host_cost[y]; });
+        const std::vector<int32_t> sorder = order_by(p->n_slices, [](int) { return 0; },
+                                                     [&](int x) { return c.host_cost[x]; });
         using Load = std::pair<int64_t, int32_t>;
         std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
         for (int b = 0; b < grid; ++b) heap.push(Load{0, b});
@@ -513,12 +525,8 @@ imrt_status make_shape(imrt_plan* p, const SellCopy& c, int k_trials, int varian
             slot_of[s] = cta_slots[l.second]++;
             heap.push(Load{l.first + c.host_cost[s], l.second});
         }
-        std::vector<int32_t> uord(n_units);
-        for (int i = 0; i < n_units; ++i) uord[i] = i;
-        std::stable_sort(uord.begin(), uord.end(), [&](int x, int y) {
-            const int cx = cta_of[us[x]], cy = cta_of[us[y]];
-            return cx != cy ? cx < cy : ucost[x] > ucost[y];
-        });
+        const std::vector<int32_t> uord = order_by(n_units, [&](int x) { return cta_of[us[x]]; },
+                                                   [&](int x) { return ucost[x]; });
         std::vector<int32_t> lsid(std::max(out->n_splits, 1), -1), cta_splits(grid, 0);
         for (int k = 0; k < n_units; ++k) {
             const int i = uord[k];
@@ -556,9 +564,7 @@ imrt_status make_shape(imrt_plan* p, const SellCopy& c, int k_trials, int varian
     }
     if (!local) {
         // global schedule: longest first over all units
-        std::vector<int32_t> ord(n_units);
-        for (int i = 0; i < n_units; ++i) ord[i] = i;
-        std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return ucost[x] > ucost[y]; });
+        const std::vector<int32_t> ord = order_by(n_units, [](int) { return 0; }, [&](int x) { return ucost[x]; });
         for (int k = 0; k < n_units; ++k) {
             recs[k] = make_rec(ord[k], usplit[ord[k]], 0);
             rec_slice[k] = us[ord[k]];
@@ -613,6 +619,15 @@ imrt_status make_shape(imrt_plan* p, const SellCopy& c, int k_trials, int varian
     TRY(dalloc(p, &U.next_unit, 1));
     CK(cudaMemsetAsync(U.ticket, 0, sizeof(int32_t), stream_of(p)));
     CK(cudaMemsetAsync(U.next_unit, 0, sizeof(int32_t), stream_of(p)));
+    CK(cudaStreamSynchronize(stream_of(p)));  // the host vectors above go out of scope
+    return IMRT_OK;
+}
+
+// The part of a forward shape that needs the beamlet-major copy and its schedule (a plan being built makes
+// its shapes before these).
+imrt_status finish_shape(imrt_plan* p, const SellCopy& c, int variant, FwdShape* out) {
+    const int grid = out->grid;
+    out->finished = true;
     // the next transposed pass's L2 prefetch pays only when its copy of D is far larger than L2
     // could hold anyway (small plans stay L2-resident, and the prefetch would delay the ticket):
     // warp w of CTA b hints the row that transposed CTA per_cta * b + w most likely takes first
@@ -625,7 +640,6 @@ imrt_status make_shape(imrt_plan* p, const SellCopy& c, int k_trials, int varian
         CK(launch_prefetch_table(p->bwd_order, p->t_seg, p->t_H, p->n, count, cap, out->pf_tab, stream_of(p)));
         out->pf_per_cta = per_cta;
     }
-    CK(cudaStreamSynchronize(stream_of(p)));  // the host vectors above go out of scope
     return IMRT_OK;
 }
 
@@ -633,14 +647,15 @@ imrt_status get_shape(imrt_plan* p, int precision, int k_trials, FwdShape** out)
     const int variant = p->opt.kernel_variant;
     auto key = std::make_tuple(precision, k_trials, variant);
     auto it = p->shapes.find(key);
+    const SellCopy& c = precision == IMRT_FP32 ? p->sell32 : p->sellq;
     if (it == p->shapes.end()) {
-        const SellCopy& c = precision == IMRT_FP32 ? p->sell32 : p->sellq;
         if (c.precision != precision)
             return set_error("plan holds no copy of D at precision %d", precision), IMRT_EINVAL;
         FwdShape sh;
         TRY(make_shape(p, c, k_trials, variant, &sh));
         it = p->shapes.emplace(key, sh).first;
     }
+    if (!it->second.finished && p->bwd_order) TRY(finish_shape(p, c, variant, &it->second));
     *out = &it->second;
     return IMRT_OK;
 }
@@ -833,7 +848,6 @@ imrt_status build_sell(imrt_plan* p, SellCopy* c, int precision, const int64_t* 
     if (!mask_out) TRY(talloc(tmask, &mask_out, p->m_pad));
     CK(launch_sell_fill(c->fmt, row_ptr, col, val, p->perm, mask_in, p->m, p->m_pad, c->slice_off, c->slice_len,
                         precision == IMRT_FP32 ? nullptr : p->inv_scale, c->val, c->col, mask_out, s));
-    CK(cudaStreamSynchronize(s));
     return IMRT_OK;
 }
 
@@ -872,6 +886,10 @@ imrt_status ensure_lambda0_rule(imrt_plan* p) {
         b.pw_lam = p->dscratch;
         void* pargs[] = {&b};
         CK(cudaLaunchKernel(power_step_kernel(), dim3(1), dim3(kBwdThreads), pargs, 0, s));
+    }
+    if (p->opt.precision != IMRT_FP32) {  // planned on the host while the passes above run
+        FwdShape* early = nullptr;
+        if (get_shape(p, p->opt.precision, 1, &early) != IMRT_OK) g_error.clear();  // as in plan_build
     }
     double lam = 0.0;
     CK(cudaMemcpyAsync(&lam, p->dscratch, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -987,6 +1005,12 @@ imrt_status plan_build(imrt_plan* p, const imrt_csr* D, const uint8_t* structure
     }
     CK(launch_transpose_fill(row_ptr, col, val, p->m, n, chunk_rows, counts, col_len, p->t_off, pair, p->t_val, p->t_row,
                              s));
+    // The host plans the forward pass's work while the GPU scatters (GB300, 61M entries in FP16: creation and
+    // one evaluation 15.0 -> 12.6 ms together with the reduced precision's plan made under the step-size
+    // rule, sorts of packed keys and the pair scatter, 0.8 ms of it). A shape
+    // that cannot be made is reported by the first call that needs it.
+    FwdShape* early = nullptr;
+    if (get_shape(p, IMRT_FP32, 1, &early) != IMRT_OK) g_error.clear();
     if (p->opt.precision != IMRT_FP32) {  // (segmented) per-beamlet scales, then the reduced voxel-major copy
         Temp tabs;
         uint32_t* absmax;
@@ -1014,7 +1038,6 @@ imrt_status plan_build(imrt_plan* p, const imrt_csr* D, const uint8_t* structure
             TRY(dalloc_bytes(p, &p->t_valq, (size_t)p->tq_entries * elem_bytes(p->opt.precision) + 64));
         CK(launch_tq_fill(p->opt.precision, p->t_off, pair, col_len, n, H, p->t_seg, p->inv_scale,
                           p->t_vals, p->t_valq, p->t_lo, s));
-        CK(cudaStreamSynchronize(s));
     }
     TRY(make_bwd_schedule(p, hlen));
     // --- structures and term coefficients (Eq. (1): c = w / |V_s|) ----------
