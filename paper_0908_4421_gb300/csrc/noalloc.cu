@@ -132,7 +132,7 @@ struct NaCoefs {
     uint32_t has_u, has_o;  // bit t: structure t has an under / over term
 };
 
-// Warp 0 of a block; the caller synchronises the block before use.
+// Warp 0 of a block; the caller has a block barrier before the first use.
 __device__ __forceinline__ void na_coefs(NaCoefs& C, const NaTerms& terms, const int32_t (*counts)[kNaMaxStruct],
                                          int count_blocks) {
     if (threadIdx.x >= 32) return;
@@ -151,19 +151,20 @@ __device__ __forceinline__ void na_coefs(NaCoefs& C, const NaTerms& terms, const
         const int c = __reduce_add_sync(0xffffffffu, part[k]);
         if (t == k) cnt = c;
     }
-    bool hu = false, ho = false;
-    if (t < kNaMaxStruct) {
-        hu = t < terms.S && !isnan(terms.Tu[t]) && terms.wu[t] != 0.0f && cnt > 0;
-        ho = t < terms.S && !isnan(terms.To[t]) && terms.wo[t] != 0.0f && cnt > 0;
-        C.Tu[t] = terms.Tu[t];
-        C.To[t] = terms.To[t];
-        C.cu[t] = hu ? (double)terms.wu[t] / (double)cnt : 0.0;
-        C.co[t] = ho ? (double)terms.wo[t] / (double)cnt : 0.0;
+    // lane k: the under-dose term of structure k, lane 8 + k its over-dose term (one FP64 division each)
+    const int k = t & 7;
+    const bool under = t < 8;
+    cnt = __shfl_sync(0xffffffffu, cnt, k);
+    const float T = under ? terms.Tu[k] : terms.To[k], w = under ? terms.wu[k] : terms.wo[k];
+    const bool has = t < 16 && k < terms.S && !isnan(T) && w != 0.0f && cnt > 0;
+    if (t < 16) {
+        (under ? C.Tu : C.To)[k] = T;
+        (under ? C.cu : C.co)[k] = has ? (double)w / (double)cnt : 0.0;
     }
-    const uint32_t bu = __ballot_sync(0xffffffffu, hu), bo = __ballot_sync(0xffffffffu, ho);
+    const uint32_t b = __ballot_sync(0xffffffffu, has);
     if (t == 0) {
-        C.has_u = bu;
-        C.has_o = bo;
+        C.has_u = b & 0xffu;
+        C.has_o = b >> 8 & 0xffu;
     }
 }
 
@@ -199,15 +200,15 @@ __device__ __forceinline__ double na_warp_sum(double v) {
 //    rows is shared by the block's 8 warps, row k to warp k mod 8, so neighbouring long rows spread over
 //    the block and the tiles over the chip. The row bounds of the next unit are loaded while the
 //    current one streams;
-//  * a lane has up to 8 columns and 8 values in flight, then their 8 gathers of x (coalesced 4-byte
+//  * a lane has up to 12 columns and 12 values in flight, then their gathers of x (coalesced 4-byte
 //    loads: rows start on any entry, and consecutive entries of a row gather neighbouring x);
 //  * the penalties of a unit are evaluated one row per lane by warp 0, from the row sums in shared
 //    memory (FP64 arithmetic is scarce: one lane doing a warp's rows in turn was a serial chain).
-// Measured on a GB300, a call: 61M entries in 305k rows 1703 -> 171 us (2.9 TB/s), 0.57M in 44k rows
-// 253 -> 53 us, against blocks of 1024 consecutive rows whose warps took 128 rows in series. Tried and
-// slower: a cp.async ring per warp over equal shares of the entries (163-202 us: a row's own cost, not
-// its entries, sets the balance), L2 prefetch of the next unit (209 us), 16 loads a lane at two or three
-// blocks an SM (185-223 us).
+// Measured on a GB300, a call: 61M entries in 305k rows 1703 -> 165 us (3.0 TB/s), 0.57M in 44k rows
+// 253 -> 42 us, against blocks of 1024 consecutive rows whose warps took 128 rows in series. Tried and
+// slower or no faster at 61M entries: a cp.async ring per warp over equal shares of the entries (163-202 us:
+// a row's own cost, not its entries, sets the balance), 16-byte loads (169-175 us), L2 prefetch of the
+// next unit (209 us), 8 loads a lane (171-185 us), 16 at three or two blocks an SM (182, 213 us).
 __global__ void __launch_bounds__(kNaThreads, kNaBlocksPerSm)
     k_na_eval(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, const float* __restrict__ val,
               int32_t m, int32_t n, int64_t nnz, const uint8_t* __restrict__ mask, const NaTerms terms,
@@ -231,10 +232,8 @@ __global__ void __launch_bounds__(kNaThreads, kNaBlocksPerSm)
     int bad = 0;
     if (blockIdx.x == 0 && tid == 0 && (row_ptr[0] != 0 || row_ptr[m] != nnz)) bad |= 1;
     imrt::pdl_wait();  // the counts and the cleared words
-    if (tid == 0) s_tile[0] = (int)gridDim.x + atomicAdd(&s->next, 1);
-    na_coefs(C, terms, s->counts, count_blocks);
-    __syncthreads();
-    int next_tile = s_tile[0], tb = 0, buf = 0;
+    na_coefs(C, terms, s->counts, count_blocks);  // (first used after the first unit's barrier)
+    int next_tile = (int)(blockIdx.x + gridDim.x), tb = 0, buf = 0;  // later tiles come from the counter
     uint32_t most = 0;  // the largest beamlet index read
     double F = 0.0;     // warp 0: this lane's rows of the tile
     const uint32_t n1 = (uint32_t)n - 1u;
@@ -246,7 +245,7 @@ __global__ void __launch_bounds__(kNaThreads, kNaBlocksPerSm)
     };
     while (tile < n_tiles) {
         const bool ends = rb + kNaUnit >= r1;  // the tile's last unit
-        if (ends && tid == 0) s_tile[tb ^ 1] = (int)gridDim.x + atomicAdd(&s->next, 1);
+        if (ends && tid == 0) s_tile[tb ^ 1] = 2 * (int)gridDim.x + atomicAdd(&s->next, 1);
         // the next unit, and the bounds of its rows
         const int n_tile = ends ? next_tile : tile;
         int n_rb = rb + kNaUnit, n_r1 = r1;
@@ -264,7 +263,7 @@ __global__ void __launch_bounds__(kNaThreads, kNaBlocksPerSm)
             la = lb = 0;
         }
         float acc[kNaRows];
-        constexpr int kU = 8;  // columns and values in flight per lane
+        constexpr int kU = 12;  // columns and values in flight per lane
 #pragma unroll
         for (int k = 0; k < kNaRows; ++k) {
             acc[k] = 0.0f;
