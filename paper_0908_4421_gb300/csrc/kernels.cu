@@ -665,7 +665,7 @@ __global__ void __launch_bounds__(kFwdThreads,
         }
         __syncthreads();
         // the CTA's objective partial of each trial: its slots added in slot order
-        if (wib < KT) {
+        if (wib < KT && (a.control || a.G_out)) {
             const int q = wib;
             Df t{0.0f, 0.0f};
             for (int i = lane; i < s_slots; i += 32) t = df_add(t, reinterpret_cast<const Df*>(lt.slots)[(size_t)i * KT + q]);
@@ -695,6 +695,9 @@ __global__ void __launch_bounds__(kFwdThreads,
     // (CTA-local schedule: once every warp of the CTA is done; issued earlier, per warp, the
     // prefetch was measured to delay the last CTAs' streaming more than it saved)
     if (!failed) prefetch_next_rows(a, s_pf, wib, lane);
+    // A dose or a pass of the step-size rule (CTA-local schedule, no controller, no objective): nothing waits
+    // for the last CTA and no counter was used, so the launch ends with its rows.
+    if (U.local && !a.control && !a.G_out) return;
     // count finished CTAs: the last one resets the schedule and, inside a solve, runs the
     // controller. Each write the controller reads was followed by a release fence of its warp
     // (x_t and the step-length partials: warp 0 in the prologue; the CTA's objective partials:
