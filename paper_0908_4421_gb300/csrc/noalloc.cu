@@ -200,15 +200,16 @@ __device__ __forceinline__ double na_warp_sum(double v) {
 //    rows is shared by the block's 8 warps, row k to warp k mod 8, so neighbouring long rows spread over
 //    the block and the tiles over the chip. The row bounds of the next unit are loaded while the
 //    current one streams;
-//  * a lane has up to 12 columns and 12 values in flight, then their gathers of x (coalesced 4-byte
-//    loads: rows start on any entry, and consecutive entries of a row gather neighbouring x);
-//  * the penalties of a unit are evaluated one row per lane by warp 0, from the row sums in shared
+//  * a lane keeps two rounds of 6 columns and 6 values: the next round of its row is in flight while the
+//    gathers of x of the current one are (coalesced 4-byte loads: rows start on any entry, and
+//    consecutive entries of a row gather neighbouring x);
+//  * the penalties of a unit are evaluated one row per lane by one warp, from the row sums in shared
 //    memory (FP64 arithmetic is scarce: one lane doing a warp's rows in turn was a serial chain).
-// Measured on a GB300, a call: 61M entries in 305k rows 1703 -> 165 us (3.0 TB/s), 0.57M in 44k rows
+// Measured on a GB300, a call: 61M entries in 305k rows 1703 -> 151 us (3.3 TB/s), 0.57M in 44k rows
 // 253 -> 42 us, against blocks of 1024 consecutive rows whose warps took 128 rows in series. Tried and
-// slower or no faster at 61M entries: a cp.async ring per warp over equal shares of the entries (163-202 us:
-// a row's own cost, not its entries, sets the balance), 16-byte loads (169-175 us), L2 prefetch of the
-// next unit (209 us), 8 loads a lane (171-185 us), 16 at three or two blocks an SM (182, 213 us).
+// slower at 61M entries: single rounds of 8 to 16 loads (165-204 us), two rounds of 4, 5 or 8 (158-171 us),
+// a cp.async ring per warp over equal shares of the entries (163-202 us: a row's own cost, not its entries,
+// sets the balance), 16-byte loads (169-175 us), L2 prefetch of the next unit (209 us).
 __global__ void __launch_bounds__(kNaThreads, kNaBlocksPerSm)
     k_na_eval(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col, const float* __restrict__ val,
               int32_t m, int32_t n, int64_t nnz, const uint8_t* __restrict__ mask, const NaTerms terms,
@@ -263,41 +264,56 @@ __global__ void __launch_bounds__(kNaThreads, kNaBlocksPerSm)
             la = lb = 0;
         }
         float acc[kNaRows];
-        constexpr int kU = 12;  // columns and values in flight per lane
+        constexpr int kU = 6;  // columns and values in flight per lane and stage
+        struct Round {
+            int32_t c[kU];
+            float v[kU];
+        };
+        // entries i, i + 32, ... of a row of `len` entries starting at c0 / v0
+        auto load = [&](Round& q, const int32_t* c0, const float* v0, int i, int len) {
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const bool in = i + 32 * u < len;
+                q.c[u] = in ? __ldcs(c0 + i + 32 * u) : 0;
+                q.v[u] = in ? __ldcs(v0 + i + 32 * u) : 0.0f;
+            }
+        };
+        auto use = [&](const Round& q, int i, int len, float& sum) {
+            float xv[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) xv[u] = x_at(q.c[u]);
+#pragma unroll
+            for (int u = 0; u < kU; ++u) sum = i + 32 * u < len && (uint32_t)q.c[u] <= n1 ? fmaf(q.v[u], xv[u], sum) : sum;
+        };
 #pragma unroll
         for (int k = 0; k < kNaRows; ++k) {
             acc[k] = 0.0f;
-            int64_t left = __shfl_sync(0xffffffffu, lb - la, k);
-            const int64_t e = __shfl_sync(0xffffffffu, la, k) + lane;
-            const int32_t* pc = col + e;
-            const float* pv = val + e;
-            int32_t c[kU];
-            float v[kU], xv[kU];
-            for (; left >= 32 * kU; left -= 32 * kU) {
-#pragma unroll
-                for (int u = 0; u < kU; ++u) {
-                    c[u] = __ldcs(pc + 32 * u);
-                    v[u] = __ldcs(pv + 32 * u);
+            int64_t a = __shfl_sync(0xffffffffu, la, k);
+            const int64_t b = __shfl_sync(0xffffffffu, lb, k);
+            while (a < b) {  // (once, but for rows longer than an int)
+                const int len = (int)min(b - a, (int64_t)1 << 30);
+                const int32_t* c0 = col + a;
+                const float* v0 = val + a;
+                a += len;
+                Round p, q;
+                int i = lane;
+                load(p, c0, v0, i, len);
+                while (true) {
+                    const int j = i + 32 * kU;
+                    if (j - lane >= len) {
+                        use(p, i, len, acc[k]);
+                        break;
+                    }
+                    load(q, c0, v0, j, len);
+                    use(p, i, len, acc[k]);
+                    i = j + 32 * kU;
+                    if (i - lane >= len) {
+                        use(q, j, len, acc[k]);
+                        break;
+                    }
+                    load(p, c0, v0, i, len);
+                    use(q, j, len, acc[k]);
                 }
-                pc += 32 * kU;
-                pv += 32 * kU;
-#pragma unroll
-                for (int u = 0; u < kU; ++u) xv[u] = x_at(c[u]);
-#pragma unroll
-                for (int u = 0; u < kU; ++u) acc[k] = (uint32_t)c[u] <= n1 ? fmaf(v[u], xv[u], acc[k]) : acc[k];
-            }
-            const int rest = (int)left - lane;  // this lane's entries: 32 u < rest
-            if (left > 0) {
-#pragma unroll
-                for (int u = 0; u < kU; ++u) {
-                    c[u] = 32 * u < rest ? __ldcs(pc + 32 * u) : 0;
-                    v[u] = 32 * u < rest ? __ldcs(pv + 32 * u) : 0.0f;
-                }
-#pragma unroll
-                for (int u = 0; u < kU; ++u) xv[u] = 32 * u < rest ? x_at(c[u]) : 0.0f;
-#pragma unroll
-                for (int u = 0; u < kU; ++u)
-                    acc[k] = 32 * u < rest && (uint32_t)c[u] <= n1 ? fmaf(v[u], xv[u], acc[k]) : acc[k];
             }
         }
 #pragma unroll

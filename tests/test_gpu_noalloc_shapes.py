@@ -1,5 +1,5 @@
 """imrt_eval_csr_noalloc at the edges of its row tiles (32 rows, 64 beyond 524,288 voxels) and of its
-loads (384 entries a round): dose and objective against FP64 sums of the same arrays."""
+loads (rounds of 192 entries, two in flight): dose and objective against FP64 sums of the same arrays."""
 import ctypes
 
 import numpy as np
@@ -37,8 +37,8 @@ def test_noalloc_row_tiles(m, n, kind):
         lengths = np.ones(m, np.int64)
     elif kind == "empty":
         lengths = np.zeros(m, np.int64)
-    elif kind == "edges":  # around a round of 384 entries
-        lengths = rng.choice([0, 1, 31, 32, 33, 383, 384, 385, 511, 512, 513], m)
+    elif kind == "edges":  # around one and two rounds of 192 entries
+        lengths = rng.choice([0, 1, 31, 32, 33, 191, 192, 193, 383, 384, 385, 513], m)
     else:
         lengths = np.where(rng.random(m) < 0.4, 0, rng.integers(0, n + 1, m))
     row_ptr, col, val = _csr(rng, m, n, lengths)
