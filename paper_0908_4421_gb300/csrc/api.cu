@@ -627,7 +627,6 @@ imrt_status make_shape(imrt_plan* p, const SellCopy& c, int k_trials, int varian
 // its shapes before these).
 imrt_status finish_shape(imrt_plan* p, const SellCopy& c, int variant, FwdShape* out) {
     const int grid = out->grid;
-    out->finished = true;
     // the next transposed pass's L2 prefetch pays only when its copy of D is far larger than L2
     // could hold anyway (small plans stay L2-resident, and the prefetch would delay the ticket):
     // warp w of CTA b hints the row that transposed CTA per_cta * b + w most likely takes first
@@ -636,10 +635,13 @@ imrt_status finish_shape(imrt_plan* p, const SellCopy& c, int variant, FwdShape*
         const int per_cta = std::min(kMaxPrefetchPerCta, (p->bwd_grid + grid - 1) / std::max(grid, 1));
         const int count = per_cta * grid;
         const int64_t cap = ((int64_t)IMRT_BWD_PREFETCH_KB * 1024 / (int64_t)(elem_bytes(c.precision) + 2)) & ~(int64_t)7;
-        TRY(dalloc(p, &out->pf_tab, (size_t)2 * count));
-        CK(launch_prefetch_table(p->bwd_order, p->t_seg, p->t_H, p->n, count, cap, out->pf_tab, stream_of(p)));
+        int64_t* tab = nullptr;
+        TRY(dalloc(p, &tab, (size_t)2 * count));
+        CK(launch_prefetch_table(p->bwd_order, p->t_seg, p->t_H, p->n, count, cap, tab, stream_of(p)));
+        out->pf_tab = tab;
         out->pf_per_cta = per_cta;
     }
+    out->finished = true;
     return IMRT_OK;
 }
 

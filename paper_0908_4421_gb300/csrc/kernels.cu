@@ -431,20 +431,30 @@ struct TrialIn {
 // (w = 0: v = 0) into shared memory, and by one CTA to v_out. Every CTA adds ||w||^2 in the
 // same fixed order (per thread, the xor tree of each warp, then the warps in order), so all
 // CTAs hold the same v and no separate update kernel runs between the passes. The squares are
-// exact and their sum a double-float (FP64 runs at a small fraction of the FP32 rate here), and one
-// thread takes the FP64 root and reciprocal: FP64 sums with the root taken by all 512 threads put 7 us
-// into every pass of the 61M-entry rule (77.5 us, now 73.7, against 70.5 us for a plain evaluation).
+// exact and their sum a double-float (FP64 runs at a small fraction of the FP32 rate here), of w scaled by a
+// power of two to at most 2 so that no square leaves the FP32 range; one thread takes the FP64 root and
+// reciprocal. FP64 sums with the root taken by all 512 threads put 7 us into every pass of the
+// 61M-entry rule (77.5 us, now about 72.5, against 70.5 us for a plain evaluation).
 __device__ __forceinline__ void power_next_x(const float* __restrict__ w, int n, int n_pad, float* xs,
                                              float* __restrict__ v_out) {
     __shared__ Df part[kFwdThreads / 32];
+    __shared__ uint32_t part_m[kFwdThreads / 32];
     __shared__ float s_inv;
     const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
-    Df ww{0.0f, 0.0f};
+    uint32_t most = 0u;  // bits of max |w|: ordered as the values are
     for (int i = tid; i < n_pad; i += kFwdThreads) {
         const float v = i < n ? __ldcg(w + i) : 0.0f;
         xs[i] = v;
-        ww = df_add(ww, df_sqr(v));
+        most = max(most, __float_as_uint(v) & 0x7fffffffu);
     }
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0) part_m[wib] = most;
+    __syncthreads();
+    for (int k = 0; k < kFwdThreads / 32; ++k) most = max(most, part_m[k]);
+    const uint32_t ex = min(max(most >> 23, 1u), 253u);          // max |w| < 2^(ex - 126)
+    const float scale = __uint_as_float((254u - ex) << 23);      // 2^(127 - ex)
+    Df ww{0.0f, 0.0f};
+    for (int i = tid; i < n_pad; i += kFwdThreads) ww = df_add(ww, df_sqr(xs[i] * scale));  // this thread's entries
     ww = warp_sum(ww);
     if (lane == 0) part[wib] = ww;
     __syncthreads();
@@ -452,7 +462,7 @@ __device__ __forceinline__ void power_next_x(const float* __restrict__ w, int n,
         Df tot = part[0];
         for (int k = 1; k < kFwdThreads / 32; ++k) tot = df_add(tot, part[k]);
         const double t = df_to_double(tot);
-        s_inv = t > 0.0 ? (float)(1.0 / sqrt(t)) : 0.0f;
+        s_inv = t > 0.0 ? (float)(1.0 / sqrt(t) * (double)scale) : 0.0f;
     }
     __syncthreads();
     const float inv = s_inv;

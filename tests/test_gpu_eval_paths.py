@@ -42,3 +42,20 @@ def test_eval_array_forms(m, n, variant):
         shared[:n] = torch.from_numpy(x)
         plan.dose(shared[:n], out=shared[:m])  # z over x
         assert np.array_equal(shared[:m].cpu().numpy(), z0)
+
+
+@pytest.mark.parametrize("exponent", [-45, -33, 0, 30, 36])
+def test_step_size_rule_scales_exactly(exponent):
+    """D scaled by a power of two scales every number of the power iteration exactly, so lambda0 times the
+    scale squared keeps its bits; the squares of the iterates reach far beyond the FP32 range."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    case = phantom.random_case(11, m=900, n=70, density=0.3, n_structures=2, empty_rows=20)
+    rules = []
+    for k in (0, exponent):
+        val = np.ldexp(case.val, k).astype(np.float32)
+        with Plan(case.row_ptr, case.col, val, case.mask, case.thresholds, case.weights, m=case.m, n=case.n) as plan:
+            rules.append(plan.info()["lambda0_rule"])
+    assert np.isfinite(rules[1]) and rules[1] > 0.0
+    assert rules[1] * 4.0 ** exponent == rules[0]
