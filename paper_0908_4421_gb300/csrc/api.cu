@@ -2379,7 +2379,7 @@ imrt_status plan_eval(imrt_plan* p, const float* x, double* G, float* z_out, flo
     // Up to two launches, no copies where the caller's arrays allow: x read in place (the kernel copies
     // whole 16-byte words of it), z written in the caller's order by the forward pass, g by the
     // transposed pass, G into mapped host memory. Before, a staging copy, an un-permute kernel, a sum
-    // kernel and two copies more. GB300, a call: dose of a 24k-voxel plan 23.4 -> 17.4 us; objective, dose and
+    // kernel and two copies more. GB300, a call: dose of a 24k-voxel plan 23.4 -> 15.7 us; objective, dose and
     // gradient of a 2M-entry plan 58.1 -> 34.1 us, of a 61M-entry one 172 -> 143 us (FP16 137 -> 111).
     const float* xs = p->v.x + (size_t)p->cur * p->n_pad;
     bool direct_z = is_device_ptr(z_out), direct_g = is_memory_of(g_out, p->device);
