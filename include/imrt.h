@@ -313,7 +313,7 @@ imrt_status plan_cancel(imrt_plan* plan);
  *               finite and >= 0, thresholds finite or NaN).
  *   x           n beamlet intensities, device.
  *   z_out       m floats, device, in the caller's row order; NULL to skip.
- *   G_out       the FP64 objective, host.
+ *   G_out       the FP64 objective, host memory (device memory takes one copy more).
  *   stream      cudaStream_t. The call waits for its stream and copies G into
  *               G_out before it returns.
  * The first call on each device looks up the scratch array's device address

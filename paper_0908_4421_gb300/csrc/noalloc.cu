@@ -427,6 +427,16 @@ bool on_device(const void* p, int dev) {
     return a.type == cudaMemoryTypeManaged;
 }
 
+// Memory that only a copy can write from the host (device memory of any GPU).
+bool needs_copy(const void* p) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice;
+}
+
 }  // namespace
 
 extern "C" imrt_status imrt_eval_csr_noalloc(const imrt_csr* D, const uint8_t* structures, int32_t n_structures,
@@ -502,14 +512,17 @@ extern "C" imrt_status imrt_eval_csr_noalloc(const imrt_csr* D, const uint8_t* s
         e = cudaLaunchKernelEx(&cfg, k_na_eval, D->row_ptr, D->col_idx, D->val, D->m, D->n, D->nnz, structures,
                                terms, x, z_out, tile_rows, n_tiles, count_blocks, s);
     }
+    // the objective and the error flag in one copy; an objective wanted in device memory takes a copy of its own
+    const bool copy_G = needs_copy(G_out);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&out, &s->res, sizeof(out), cudaMemcpyDeviceToHost, cs);
+    if (e == cudaSuccess && copy_G) e = cudaMemcpyAsync(G_out, &s->res.G, sizeof(double), cudaMemcpyDefault, cs);
     if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
     if (e != cudaSuccess) {
         na_set_error("CUDA error: %s", cudaGetErrorString(e));
         return IMRT_ECUDA;
     }
     const int32_t bad = out.bad;
-    *G_out = out.G;
+    if (!copy_G) *G_out = out.G;
     if (bad) {
         na_set_error("invalid CSR: %s%s%s", (bad & 1) ? "row offsets outside [0, nnz] or decreasing" : "",
                      (bad & 3) == 3 ? "; " : "", (bad & 2) ? "beamlet index outside [0, n)" : "");
