@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "../../include/imrt.h"
+#include "host_rules.h"
 #include "imrt_internal.cuh"
 
 using namespace imrt;
@@ -56,24 +57,37 @@ void set_error(const char* fmt, ...) {
 
 inline int64_t round_up(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 
-bool is_device_ptr(const void* p) {
-    if (!p) return false;
+// Where p lives, and the device that owns it.
+Memory memory_of(const void* p, int* owner) {
     cudaPointerAttributes attr;
+    *owner = -1;
+    if (!p) return Memory::kHost;
     if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return Memory::kHost;
     }
-    return attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged;
+    *owner = attr.device;
+    return attr.type == cudaMemoryTypeDevice ? Memory::kDevice
+           : attr.type == cudaMemoryTypeManaged ? Memory::kManaged
+                                                : Memory::kHost;
+}
+
+bool is_device_ptr(const void* p) {
+    int owner;
+    return memory_of(p, &owner) != Memory::kHost;
+}
+
+// Memory that kernels on device `dev` may use in place (kernels_may_use).
+bool usable_on(const void* p, int dev) {
+    int owner;
+    const Memory where = memory_of(p, &owner);
+    return kernels_may_use(where, owner, dev);
 }
 
 // Device memory of device `dev` itself (not managed, not another GPU's).
 bool is_memory_of(const void* p, int dev) {
-    cudaPointerAttributes attr;
-    if (!p || cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return attr.type == cudaMemoryTypeDevice && attr.device == dev;
+    int owner;
+    return memory_of(p, &owner) == Memory::kDevice && owner == dev;
 }
 
 // Whether the float arrays a (na entries) and b (nb entries) share memory.
@@ -938,10 +952,10 @@ imrt_status plan_build(imrt_plan* p, const imrt_csr* D, const uint8_t* structure
             return set_error("row_ptr[0] must be 0 and row_ptr[m] must equal nnz"), IMRT_EINVAL;
     }
     const uint8_t* mask_in = structures;
-    if (!is_device_ptr(structures)) {
+    if (!usable_on(structures, p->device)) {
         uint8_t* dm;
         TRY(talloc(tmaskin, &dm, m));
-        CK(cudaMemcpyAsync(dm, structures, m, cudaMemcpyHostToDevice, s));
+        CK(cudaMemcpyAsync(dm, structures, m, cudaMemcpyDefault, s));
         mask_in = dm;
     }
     // --- validation and row lengths ----------------------------------------
@@ -2382,7 +2396,7 @@ imrt_status plan_eval(imrt_plan* p, const float* x, double* G, float* z_out, flo
     // kernel and two copies more. GB300, a call: dose of a 24k-voxel plan 23.4 -> 15.7 us; objective, dose and
     // gradient of a 2M-entry plan 58.1 -> 34.1 us, of a 61M-entry one 172 -> 143 us (FP16 137 -> 111).
     const float* xs = p->v.x + (size_t)p->cur * p->n_pad;
-    bool direct_z = is_device_ptr(z_out), direct_g = is_memory_of(g_out, p->device);
+    bool direct_z = usable_on(z_out, p->device), direct_g = is_memory_of(g_out, p->device);
     if (overlap(z_out, p->m, g_out, p->n)) direct_z = direct_g = false;  // z is written last
     if (x) {
         const bool in_place = (p->n & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0 &&
