@@ -20,6 +20,7 @@
 //                the stop test, and the CUDA-graph loop condition.
 //   k_init / k_finish  x_1 and the KKT residual.
 #include "stream.cuh"
+#include "wide_sum.cuh"
 
 namespace imrt {
 
@@ -429,16 +430,30 @@ struct TrialIn {
 
 // The power iteration's next vector inside the forward pass that uses it: v = w / ||w||
 // (w = 0: v = 0) into shared memory, and by one CTA to v_out. Every CTA adds ||w||^2 in the
-// same fixed order (per thread, the xor tree of each warp, then the warps in order), so all
-// CTAs hold the same v and no separate update kernel runs between the passes. The squares are
-// exact and their sum a double-float (FP64 runs at a small fraction of the FP32 rate here), of w scaled by a
-// power of two to at most 2 so that no square leaves the FP32 range; one thread takes the FP64 root and
-// reciprocal. FP64 sums with the root taken by all 512 threads put 7 us into every pass of the
-// 61M-entry rule (77.5 us, now about 72.5, against 70.5 us for a plain evaluation).
+// same fixed order (per thread, the xor tree of each warp, then that of the 16 warps' sums), so
+// all CTAs hold the same v and no separate update kernel runs between the passes. The sum is held in three
+// floats (wide_sum.cuh): over 70 to 28,000 entries at most 1.0 unit of 2^-53 from the exact sum, where an FP64
+// sum in the same order was up to 4.3 off and a double-float one up to 85. w is scaled by a power of two, to
+// below 4, so that no square leaves the FP32 range; one thread takes the FP64 root and reciprocal (FP64 sums with
+// the root taken by all 512 threads put 7 us into every pass of the 61M-entry rule).
+__device__ __forceinline__ WideSum warp_sum(WideSum v, int first) {  // xor tree from distance `first` down
+#pragma unroll
+    for (int o = first; o > 0; o >>= 1) {
+        WideSum w;
+        w.a = __shfl_xor_sync(0xffffffffu, v.a, o);
+        w.b = __shfl_xor_sync(0xffffffffu, v.b, o);
+        w.c = __shfl_xor_sync(0xffffffffu, v.c, o);
+        v = wide_add(v, w);
+    }
+    return v;
+}
+
 __device__ __forceinline__ void power_next_x(const float* __restrict__ w, int n, int n_pad, float* xs,
                                              float* __restrict__ v_out) {
-    __shared__ Df part[kFwdThreads / 32];
-    __shared__ uint32_t part_m[kFwdThreads / 32];
+    constexpr int kWarps = kFwdThreads / 32;
+    static_assert(kWarps == 16, "the warps' sums are added by a tree over 16 lanes");
+    __shared__ WideSum part[kWarps];
+    __shared__ uint32_t part_m[kWarps];
     __shared__ float s_inv;
     const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
     uint32_t most = 0u;  // bits of max |w|: ordered as the values are
@@ -450,19 +465,17 @@ __device__ __forceinline__ void power_next_x(const float* __restrict__ w, int n,
     most = __reduce_max_sync(0xffffffffu, most);
     if (lane == 0) part_m[wib] = most;
     __syncthreads();
-    for (int k = 0; k < kFwdThreads / 32; ++k) most = max(most, part_m[k]);
-    const uint32_t ex = min(max(most >> 23, 1u), 253u);          // max |w| < 2^(ex - 126)
+    for (int k = 0; k < kWarps; ++k) most = max(most, part_m[k]);
+    const uint32_t ex = min(max(most >> 23, 1u), 253u);          // max |w| < 2^(ex - 126), or 2^128
     const float scale = __uint_as_float((254u - ex) << 23);      // 2^(127 - ex)
-    Df ww{0.0f, 0.0f};
-    for (int i = tid; i < n_pad; i += kFwdThreads) ww = df_add(ww, df_sqr(xs[i] * scale));  // this thread's entries
-    ww = warp_sum(ww);
+    WideSum ww{0.0f, 0.0f, 0.0f};
+    for (int i = tid; i < n_pad; i += kFwdThreads) ww = wide_add(ww, wide_square(xs[i] * scale));  // this thread's entries
+    ww = warp_sum(ww, 16);
     if (lane == 0) part[wib] = ww;
     __syncthreads();
-    if (tid == 0) {
-        Df tot = part[0];
-        for (int k = 1; k < kFwdThreads / 32; ++k) tot = df_add(tot, part[k]);
-        const double t = df_to_double(tot);
-        s_inv = t > 0.0 ? (float)(1.0 / sqrt(t) * (double)scale) : 0.0f;
+    if (wib == 0) {
+        const double t = wide_to_double(warp_sum(part[lane & (kWarps - 1)], kWarps / 2));
+        if (lane == 0) s_inv = t > 0.0 ? (float)(1.0 / sqrt(t) * (double)scale) : 0.0f;
     }
     __syncthreads();
     const float inv = s_inv;
