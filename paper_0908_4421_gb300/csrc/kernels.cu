@@ -61,8 +61,10 @@ struct CtlStage {
     SolveParams P;
 };
 
+// Not inlined: inside the bulk-copy kernel its code made the consumers' loop slower (305k voxels, a forward pass:
+// 92.7 us inlined, 90.2 us called; 91.5 us with the CTA-wide tree it replaced). The call itself does not show.
 template <int KT>
-__device__ void control_step(int phase, DevState* st, const Vecs& v, const FwdUnits& U, int n, int grid,
+__device__ __noinline__ void control_step(int phase, DevState* st, const Vecs& v, const FwdUnits& U, int n, int grid,
                              CtlStage& cs, int cancel_req) {
     DevState& S = cs.S;
     const SolveParams& P = cs.P;
@@ -75,27 +77,36 @@ __device__ void control_step(int phase, DevState* st, const Vecs& v, const FwdUn
     // One warp adds one sum whole (G of a step size, or its ||x_t - x||^2): every lane's loads in flight
     // at once, its values in order, then the xor tree. No second level over the warps: its 16 dependent
     // FP64 additions were as long as the rest (FP64 is slow here). GB300: 200 iterations of a 24k-voxel
-    // plan 2.92 -> 2.78 ms, of the 61M-entry plan 26.32 -> 26.18 ms.
+    // plan 2.92 -> 2.78 ms, of the 61M-entry plan 26.32 -> 26.18 ms. That is one partial a CTA; the device-wide
+    // schedules leave one per 1,024 voxels, where one warp would walk serial rounds. Beyond kCtlRun partials (one
+    // round of a warp's loads) G is cut into equal runs, a warp each, added in run order. A forward pass on a GB300,
+    // one warp -> runs: 3,907 partials (4M voxels) 178.7 -> 170.3 us, 977 partials 56.4 -> 54.9 us, in the bulk-copy
+    // kernel 191.8 -> 185.8 us.
+    constexpr int kCtlRun = 256, kCtlRuns = 8;
     int status_now = 0;
     if (tid == 0) status_now = __ldcg(&st->status);
     // ||g(x_1)||_inf is taken once, at the first trial pass (S is uniform over the CTA)
     const bool want_g1 = phase == 1 && !S.g1_done;
-    for (int t = wib; t < (phase == 0 ? nq : 2 * nq); t += nw) {
-        const bool is_d = t >= nq;
-        const int q = is_d ? t - nq : t, count = is_d ? grid : U.n_obj;
+    __shared__ double run_sum[kMaxTrials][kCtlRuns];
+    const int runs = max(1, min(kCtlRuns, (U.n_obj + kCtlRun - 1) / kCtlRun));
+    for (int t = wib; t < nq * runs + (phase == 0 ? 0 : nq); t += nw) {
+        const bool is_d = t >= nq * runs;
+        const int q = is_d ? t - nq * runs : t / runs, run = is_d ? 0 : t - q * runs;
+        const int per = (U.n_obj + runs - 1) / runs;
+        const int i0 = is_d ? 0 : min(U.n_obj, run * per), i1 = is_d ? grid : min(U.n_obj, i0 + per);
         const double* src = is_d ? v.dpart + (size_t)q * grid : U.obj + (size_t)q * U.n_obj;
         constexpr int kL = 8;
         double sum = 0.0;
-        for (int i = lane; i < count; i += 32 * kL) {
+        for (int i = i0 + lane; i < i1; i += 32 * kL) {
             double d[kL];
 #pragma unroll
-            for (int u = 0; u < kL; ++u) d[u] = i + 32 * u < count ? __ldcg(src + i + 32 * u) : 0.0;
+            for (int u = 0; u < kL; ++u) d[u] = i + 32 * u < i1 ? __ldcg(src + i + 32 * u) : 0.0;
 #pragma unroll
             for (int u = 0; u < kL; ++u)
-                if ((i - lane) + 32 * u < count) sum += d[u];  // (uniform: no FP64 work past the end)
+                if ((i - lane) + 32 * u < i1) sum += d[u];  // (uniform: no FP64 work past the end)
         }
         sum = warp_sum(sum);
-        if (lane == 0) sums[is_d ? kMaxTrials + q : q] = sum;
+        if (lane == 0) (is_d ? sums[kMaxTrials + q] : runs == 1 ? sums[q] : run_sum[q][run]) = sum;
     }
     if (want_g1) {
         float ginf = 0.0f;
@@ -112,6 +123,14 @@ __device__ void control_step(int phase, DevState* st, const Vecs& v, const FwdUn
     }
     if (tid == 0) S.status = status_now;
     __syncthreads();
+    if (runs > 1) {
+        if (tid < nq) {
+            double t = 0.0;
+            for (int k = 0; k < runs; ++k) t += run_sum[tid][k];
+            sums[tid] = t;
+        }
+        __syncthreads();
+    }
     if (want_g1 && tid == 0) {
         float t = 0.0f;
         for (int k = 0; k < nw; ++k) t = fmaxf(t, shf[k]);
