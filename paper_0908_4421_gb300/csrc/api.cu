@@ -983,13 +983,7 @@ imrt_status plan_build(imrt_plan* p, const imrt_csr* D, const uint8_t* structure
     CK(launch_sigma_sort(len, m, p->m_pad, p->perm, s));
     TRY(build_sell(p, &p->sell32, IMRT_FP32, row_ptr, col, val, len, mask_in, s));
     // --- beamlet-major copy -------------------------------------------------
-    // chunks small enough to keep the GPU's SMs evenly busy (the rows of one chunk are one CTA's
-    // work, and long rows lie together): 512 rows to start with, halved down to 32 while there are
-    // fewer than eight chunks an SM. Measured count + scan + scatter: 24k voxels 124 us at 512 rows, 23 us
-    // at 32; 305k voxels (61M entries) 2.08 ms at 512 rows, 2.03 ms at 128.
-    int chunk_rows = kTChunkRows;
-    while (chunk_rows > 32 && (p->m + chunk_rows - 1) / chunk_rows < 8 * p->sm_count) chunk_rows /= 2;
-    while ((int64_t)((p->m + chunk_rows - 1) / chunk_rows) * n * 4 > kTCountBytes && chunk_rows < p->m) chunk_rows *= 2;
+    const int chunk_rows = transpose_chunk_rows(p->m, n, p->sm_count);
     const int n_chunks = (p->m + chunk_rows - 1) / chunk_rows;
     Temp tcounts, tcl, tpad;
     int32_t* counts;

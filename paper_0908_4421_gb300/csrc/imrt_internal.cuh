@@ -46,11 +46,7 @@ constexpr int kMaxPrefetchPerCta = 8;  // forward CTA's L2 prefetch targets (tra
 #ifndef IMRT_BWD_PREFETCH_KB
 #define IMRT_BWD_PREFETCH_KB 64  // forward tail: L2 prefetch (KB per row) of the next transposed pass's first rows
 #endif
-// Beamlet-major build: voxel rows per counting-sort chunk (doubled while the chunk x beamlet
-// count table would exceed kTCountBytes).
-constexpr int kTChunkRows = 512;
 constexpr int kMaxSegments = 16;  // of 65536 voxels, in a segmented beamlet-major copy
-constexpr int64_t kTCountBytes = 256ll << 20;
 constexpr int kCtlThreads = 256;
 constexpr int kTmaMaxConsumers = 8;   // bulk-copy forward kernel: 1 producer + up to 8 consumer warps
 constexpr int kTmaThreads = 32 * (1 + kTmaMaxConsumers);

@@ -62,12 +62,20 @@ class ServeResult:
         return self.done - self.arrival
 
 
+def count_table_bytes(m: int, n: int) -> int:
+    """Upper bound, for any number of SMs, of the beamlet-major build's count table (csrc/host_rules.h): one
+    32-bit word per beamlet and chunk of 512 rows up to 256 MiB, of down to 32 rows up to 32 MiB."""
+    def table(rows):
+        return -(-m // rows) * n * 4
+    return max(min(table(512), 256 << 20), min(table(32), 32 << 20))
+
+
 def plan_footprint_bytes(m: int, n: int, nnz: int, precision: int) -> int:
     """Upper estimate of a plan's device memory before it exists (both FP32 copies of D, a reduced
-    copy, 9 buffer sets of x / z / r, build temporaries); replaced by the measured size once built."""
+    copy, 9 buffer sets of x / r, build temporaries); replaced by the measured size once built."""
     per_nnz = 8 * 1.05 + 8 + (8 if precision != L.FP32 else 0) + 12  # + build temporaries (CSR copy)
     m_pad = (m + 31) // 32 * 32
-    return int(nnz * per_nnz + m_pad * (9 * 8 + 24) + n * 200 + (64 << 20))
+    return int(nnz * per_nnz + m_pad * (9 * 4 + 44) + n * 200 + count_table_bytes(m, n) + (64 << 20))
 
 
 class _Request:

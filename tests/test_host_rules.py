@@ -12,6 +12,8 @@ WRAPPERS = """
 extern "C" int may_use(int where, int owner, int dev) {
     return imrt::kernels_may_use(static_cast<imrt::Memory>(where), owner, dev);
 }
+extern "C" int chunk_rows(int m, int n, int sm_count) { return imrt::transpose_chunk_rows(m, n, sm_count); }
+extern "C" long long table_bytes(int m, int n, int rows) { return imrt::count_table_bytes(m, n, rows); }
 """
 
 
@@ -39,3 +41,18 @@ def test_every_array_of_a_caller_that_a_kernel_takes_in_place_passes_the_rule():
     assert "direct_g = is_memory_of(g_out, p->device)" in text
     assert "is_memory_of(x, p->device)" in text
     assert "usable_on(structures, p->device)" in text
+
+
+@pytest.mark.parametrize("n", [1, 620, 3140, 20000, 28000])
+@pytest.mark.parametrize("m", [1, 31, 2000, 24000, 100000, 305000, 1048576, 16777216, 2 ** 31 - 1025])
+def test_count_table_stays_within_the_admission_estimate(rules, m, n):
+    from paper_0908_4421_gb300 import serve
+    rules.table_bytes.restype = ctypes.c_longlong
+    coarse = min(rules.table_bytes(m, n, 512), 256 << 20)
+    for sm_count in (1, 76, 152, 4096):
+        rows = rules.chunk_rows(m, n, sm_count)
+        table = rules.table_bytes(m, n, rows)
+        assert rows >= 32 and rows & (rows - 1) == 0
+        # smaller chunks never cost more than 32 MiB beyond what chunks of 512 rows take
+        assert table <= max(coarse, 32 << 20)
+        assert table <= serve.count_table_bytes(m, n) <= serve.plan_footprint_bytes(m, n, 0, 0) - (64 << 20)
