@@ -659,6 +659,22 @@ imrt_status finish_shape(imrt_plan* p, const SellCopy& c, int variant, FwdShape*
     return IMRT_OK;
 }
 
+// Runs make() and, if it fails, gives back the device memory it took: a step that each later call would try
+// again must not leave its part on the plan every time.
+template <class M>
+imrt_status all_or_nothing(imrt_plan* p, M&& make) {
+    const size_t kept = p->allocations.size();
+    const int64_t bytes = p->device_bytes;
+    const imrt_status st = make();
+    if (st == IMRT_OK) return st;
+    while (p->allocations.size() > kept) {
+        cudaFreeAsync(p->allocations.back(), stream_of(p));
+        p->allocations.pop_back();
+    }
+    p->device_bytes = bytes;
+    return st;
+}
+
 imrt_status get_shape(imrt_plan* p, int precision, int k_trials, FwdShape** out) {
     const int variant = p->opt.kernel_variant;
     auto key = std::make_tuple(precision, k_trials, variant);
@@ -668,10 +684,11 @@ imrt_status get_shape(imrt_plan* p, int precision, int k_trials, FwdShape** out)
         if (c.precision != precision)
             return set_error("plan holds no copy of D at precision %d", precision), IMRT_EINVAL;
         FwdShape sh;
-        TRY(make_shape(p, c, k_trials, variant, &sh));
+        TRY(all_or_nothing(p, [&] { return make_shape(p, c, k_trials, variant, &sh); }));
         it = p->shapes.emplace(key, sh).first;
     }
-    if (!it->second.finished && p->bwd_order) TRY(finish_shape(p, c, variant, &it->second));
+    if (!it->second.finished && p->bwd_order)
+        TRY(all_or_nothing(p, [&] { return finish_shape(p, c, variant, &it->second); }));
     *out = &it->second;
     return IMRT_OK;
 }
@@ -686,7 +703,7 @@ FwdArgs fwd_args(imrt_plan* p, const SellCopy& c, const FwdShape& sh, int mode) 
     a.stages = sh.stages;
     a.mask = p->mask;
     a.r_index = p->perm;
-    if (sh.pf_tab) {  // the next transposed pass's first rows, hinted into L2 (make_shape)
+    if (sh.pf_tab) {  // the next transposed pass's first rows, hinted into L2 (finish_shape)
         a.nx_tab = sh.pf_tab;
         a.nx_val = c.precision != IMRT_FP32 ? (const void*)p->t_valq : (const void*)p->t_vals;
         a.nx_lo = p->t_lo;
@@ -903,7 +920,11 @@ imrt_status ensure_lambda0_rule(imrt_plan* p) {
         void* pargs[] = {&b};
         CK(cudaLaunchKernel(power_step_kernel(), dim3(1), dim3(kBwdThreads), pargs, 0, s));
     }
-    if (p->opt.precision != IMRT_FP32) {  // planned on the host while the passes above run
+    // A plan of the graph solver needs the reduced precision's forward pass for every solve and evaluation: it is
+    // planned on the host while the passes above run (creation of a 61M-entry FP16 plan and one evaluation 14.1 ->
+    // 12.3 ms). The team solver never launches it, and there the uploads after the rule only add round trips
+    // (plan_update of a 127k-entry plan 1041 us without, 1066 us with it; of a 61M-entry one 9.44 and 9.57 ms).
+    if (p->opt.precision != IMRT_FP32 && p->opt.solver == IMRT_SOLVER_GRAPH) {
         FwdShape* early = nullptr;
         if (get_shape(p, p->opt.precision, 1, &early) != IMRT_OK) g_error.clear();  // as in plan_build
     }
@@ -1015,12 +1036,15 @@ imrt_status plan_build(imrt_plan* p, const imrt_csr* D, const uint8_t* structure
     }
     CK(launch_transpose_fill(row_ptr, col, val, p->m, n, chunk_rows, counts, col_len, p->t_off, pair, p->t_val, p->t_row,
                              s));
-    // The host plans the forward pass's work while the GPU scatters (GB300, 61M entries in FP16: creation and
-    // one evaluation 15.0 -> 12.6 ms together with the reduced precision's plan made under the step-size
-    // rule, sorts of packed keys and the pair scatter, 0.8 ms of it). A shape
-    // that cannot be made is reported by the first call that needs it.
-    FwdShape* early = nullptr;
-    if (get_shape(p, IMRT_FP32, 1, &early) != IMRT_OK) g_error.clear();
+    // The host plans the FP32 forward pass's work while the GPU scatters, if this plan's creation or solves run
+    // it (creation of a 61M-entry FP16 plan and one evaluation 15.1 -> 14.1 ms). A shape that cannot be made is
+    // reported by the first call that needs it.
+    bool under = false;  // (the x_init = 0 rule evaluates D 1)
+    for (int st = 0; st < p->S; ++st) under = under || (!std::isnan(thresholds[2 * st]) && weights[2 * st] != 0.0f);
+    if (under || p->opt.lambda0 <= 0.0 || (p->opt.precision == IMRT_FP32 && p->opt.solver == IMRT_SOLVER_GRAPH)) {
+        FwdShape* early = nullptr;
+        if (get_shape(p, IMRT_FP32, 1, &early) != IMRT_OK) g_error.clear();
+    }
     if (p->opt.precision != IMRT_FP32) {  // (segmented) per-beamlet scales, then the reduced voxel-major copy
         Temp tabs;
         uint32_t* absmax;
