@@ -157,7 +157,8 @@ typedef struct {
     int64_t nnz;
     int64_t sell_entries;      /* stored (padded) entries of the voxel-major copy */
     int64_t t_entries;         /* stored (padded) entries of the beamlet-major copy */
-    int64_t fwd_bytes;         /* algorithmic bytes of one forward pass (CSR-equivalent) */
+    int64_t fwd_bytes;         /* algorithmic bytes of one forward pass of a solve (CSR-equivalent; an
+                                  evaluation that returns the dose writes 4 m more) */
     int64_t bwd_bytes;         /* algorithmic bytes of one transposed pass */
     int64_t device_bytes;      /* device memory held by the plan */
     int32_t fwd_grid, fwd_block, bwd_grid, bwd_block;

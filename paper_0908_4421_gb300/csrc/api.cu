@@ -756,13 +756,13 @@ const SellCopy& copy_of(const imrt_plan* p, int precision) {
     return precision == IMRT_FP32 ? p->sell32 : p->sellq;
 }
 
-// CSR-equivalent algorithmic bytes of one forward and one transposed pass at `precision`:
-// values + indices + row offsets + x + (z and r writes; mask and r-order reads) forward;
+// CSR-equivalent algorithmic bytes of one forward and one transposed pass of a solve at `precision`:
+// values + indices + row offsets + x + 9 a voxel (r write; mask and r-order reads; no dose is stored) forward;
 // values + voxel indices (16-bit inside segments, else int32) + row or segment offsets + r + g.
 void pass_bytes(const imrt_plan* p, int precision, int64_t* fwd, int64_t* bwd) {
     const SellCopy& c = copy_of(p, precision);
     const int64_t vb = (int64_t)elem_bytes(precision), cb = c.fmt == IMRT_FP32 ? 4 : 2;
-    *fwd = p->nnz * (vb + cb) + (int64_t)(p->m + 1) * 8 + (int64_t)p->n * 4 + (int64_t)p->m * 13;
+    *fwd = p->nnz * (vb + cb) + (int64_t)(p->m + 1) * 8 + (int64_t)p->n * 4 + (int64_t)p->m * 9;
     *bwd = p->t_H == 0 ? p->nnz * (vb + 4) + (int64_t)(p->n + 1) * 8 + (int64_t)p->m * 4 + (int64_t)p->n * 4
                        : p->nnz * (vb + 2) + ((int64_t)p->n * p->t_H + 1) * 8 + (int64_t)p->m * 4 +
                              (int64_t)p->n * 4;
