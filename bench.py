@@ -50,7 +50,8 @@ def measured_peaks():
         return 6800.0, "fallback"
 
 
-SOURCE_FILES = ("kernels.cu", "stream.cuh", "team.cu", "imrt_internal.cuh", "ptx.cuh", "format.cu", "api.cu")
+SOURCE_FILES = ("kernels.cu", "stream.cuh", "team.cu", "imrt_internal.cuh", "ptx.cuh", "format.cu", "api.cu",
+                "noalloc.cu", "host_rules.h", "wide_sum.cuh")
 
 
 def kernel_source_hash() -> str:
