@@ -305,32 +305,9 @@ __device__ __forceinline__ void store_t(const TDest& o, int64_t k, float v, int3
     }
 }
 
-// Pass 3: scatter. Rows of a chunk are visited in order, so each beamlet row
-// receives voxels in ascending (caller) index; within one voxel row the
-// columns are distinct, so the per-beamlet cursors need no atomics.
-template <bool PAIR>
-__global__ void k_t_scatter(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
-                            const float* __restrict__ val, int32_t m, int32_t n, int32_t chunk_rows,
-                            const int32_t* __restrict__ counts, const int64_t* __restrict__ t_off, TDest out) {
-    extern __shared__ int32_t cursor[];
-    for (int c = threadIdx.x; c < n; c += blockDim.x) cursor[c] = counts[(size_t)blockIdx.x * n + c];
-    __syncthreads();
-    // the caller's voxel order: it keeps a beamlet's voxels close together in r, which the
-    // transposed pass gathers (the SELL permutation scatters them inside each sorting window)
-    const int j0 = blockIdx.x * chunk_rows, j1 = min(m, j0 + chunk_rows);
-    for (int j = j0; j < j1; ++j) {
-        for (int64_t k = row_ptr[j] + threadIdx.x; k < row_ptr[j + 1]; k += blockDim.x) {
-            const int c = col[k];
-            const int pos = cursor[c];
-            cursor[c] = pos + 1;
-            store_t<PAIR>(out, t_off[c] + pos, val[k], j);
-        }
-        __syncthreads();
-    }
-}
-
-// Pass 3, 32 voxel rows at a time (the same output as k_t_scatter). Step a: every entry of the
-// block's rows sets its row's bit in its beamlet's mask. Step b: an entry's position in its
+// Pass 3: scatter, 32 voxel rows at a time in the caller's voxel order (it keeps a beamlet's voxels close
+// together in r, which the transposed pass gathers; the SELL permutation scatters them inside each sorting
+// window). Step a: every entry of the block's rows sets its row's bit in its beamlet's mask. Step b: an entry's position in its
 // beamlet row is the beamlet's cursor plus the number of the block's lower rows holding that
 // beamlet (the mask bits below its own), so each beamlet row still receives its voxels in
 // ascending index, with no ordering between the threads. Step c: each cursor advances by its
@@ -339,7 +316,7 @@ __global__ void k_t_scatter(const int64_t* __restrict__ row_ptr, const int32_t* 
 // measured slower: every range re-reads the column indices.)
 constexpr int kTBlockRows = 32;
 template <bool PAIR>
-__global__ void k_t_scatter_blocks(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+__global__ void k_t_scatter(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
                                    const float* __restrict__ val, int32_t m, int32_t n, int32_t chunk_rows,
                                    const int32_t* __restrict__ counts, const int64_t* __restrict__ t_off, TDest out) {
     extern __shared__ int32_t cursor[];                      // n: position within the beamlet row
@@ -695,23 +672,16 @@ cudaError_t launch_transpose_fill(const int64_t* row_ptr, const int32_t* col, co
                                   cudaStream_t stream) {
     const TDest out{pair, t_val, t_row};
     const int n_chunks = (m + chunk_rows - 1) / chunk_rows;
-    int dev = 0, max_smem = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e != cudaSuccess) return e;
-    // the row-block scatter keeps a cursor and a mask per beamlet in shared memory; beyond that
-    // room, the row-by-row scatter (a cursor per beamlet) gives the same copy
-    const size_t smem2 = (size_t)n * 2 * sizeof(int32_t);
-    const bool blocks = smem2 + 1024 <= (size_t)max_smem;
-    const size_t smem = blocks ? smem2 : (size_t)n * sizeof(int32_t);
+    // a cursor and a mask per beamlet in shared memory: plans hold x and g there, which is as much (set_sizes)
+    const size_t smem = (size_t)n * 2 * sizeof(int32_t);
     auto launch = [&](auto kernel) {
         cudaError_t r = smem > 48 * 1024 ? set_max_dynamic_smem(kernel) : cudaSuccess;
         if (r != cudaSuccess) return r;
         kernel<<<n_chunks, 256, smem, stream>>>(row_ptr, col, val, m, n, chunk_rows, counts, t_off, out);
         return cudaGetLastError();
     };
-    if (pair) return blocks ? launch(k_t_scatter_blocks<true>) : launch(k_t_scatter<true>);
-    e = blocks ? launch(k_t_scatter_blocks<false>) : launch(k_t_scatter<false>);
+    if (pair) return launch(k_t_scatter<true>);
+    const cudaError_t e = launch(k_t_scatter<false>);
     if (e != cudaSuccess) return e;
     k_t_pad<<<blocks_for(n, 256), 256, 0, stream>>>(col_len, t_off, n, t_val, t_row);
     return cudaGetLastError();

@@ -1062,9 +1062,9 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_forward_tma(const FwdArgs a)
         for (int q = 0; q < KT; ++q) {
             if (mode == kFwdTrial) {
                 const int set = (cur + 1 + q) % kSets;
-                    rq[q] = a.v.r + (size_t)set * a.m_pad;
+                rq[q] = a.v.r + (size_t)set * a.m_pad;
             } else {
-                    rq[q] = a.r_dst ? a.r_dst : a.v.r + (size_t)st->cur * a.m_pad;
+                rq[q] = a.r_dst ? a.r_dst : a.v.r + (size_t)st->cur * a.m_pad;
             }
         }
         float acc[KT];

@@ -80,7 +80,9 @@ struct NaTerms {
 // Structure voxel counts, one set per block (every block writes its own, so nothing has to be
 // cleared first), and the words of the scratch that k_na_eval needs at zero. A thread counts
 // eight structures of up to 255 mask bytes in the bytes of two words (bit t of a mask byte is
-// spread to byte t), so the loop has no atomics.
+// spread to byte t), so the loop has no atomics. 32 blocks, so that one lane a block reads them back in one
+// round trip; the evaluation waits for them, which the largest sizes notice (1M voxels with 4 entries each: a
+// call 572 -> 253 us with both kernels rewritten, 16.7M: 7.17 -> 3.88 ms, of which the counts 0.18 ms).
 __global__ void __launch_bounds__(kNaThreads) k_na_counts(const uint8_t* __restrict__ mask, int32_t m, NaScratch* s) {
     __shared__ int32_t local[kNaMaxStruct];
     imrt::pdl_launch_dependents();  // k_na_eval reads what this writes after its own wait

@@ -118,8 +118,7 @@ __device__ __forceinline__ void cta_sum(Df (&v)[NQ], CtaRed& red, double* out) {
 }
 
 // The busy slices' part of G for every evaluated step size: their partials (double-float pairs,
-// stored by unit index) added in unit order
-// (their sums per warp, into red).
+// stored by unit index), per thread in unit order and summed per warp into red; cta_sum_final adds the warps.
 template <int NQ>
 __device__ __forceinline__ void sum_objective(const TeamPlan& P, const double* objb, int nq, CtaRed& red) {
     const bool multi = P.team_size > 1;
