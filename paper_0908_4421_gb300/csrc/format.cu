@@ -449,10 +449,13 @@ __global__ void __launch_bounds__(256) k_tq_fill(const int64_t* __restrict__ t_o
         const int64_t f = src[h] + (ps - sb[h]) + ((e - ps) >> 3);
         float v[8];
         uint32_t lo[8];
+        // a padding entry (value 0) names the run's last voxel: r is written there in every pass, which it is
+        // not at voxels without entries
+        const uint32_t pad = f + 7 * sg < src[h + 1] ? 0u : __ldg(pair + src[h + 1] - 1).y;
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
             const bool in = f + t * sg < src[h + 1];
-            const uint2 w = in ? __ldg(pair + f + t * sg) : make_uint2(0u, 0u);
+            const uint2 w = in ? __ldg(pair + f + t * sg) : make_uint2(0u, pad);
             v[t] = __uint_as_float(w.x);
             lo[t] = w.y & 0xffffu;
         }
