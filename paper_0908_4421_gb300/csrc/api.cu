@@ -920,11 +920,11 @@ imrt_status ensure_lambda0_rule(imrt_plan* p) {
         void* pargs[] = {&b};
         CK(cudaLaunchKernel(power_step_kernel(), dim3(1), dim3(kBwdThreads), pargs, 0, s));
     }
-    // A plan of the graph solver needs the reduced precision's forward pass for every solve and evaluation: it is
-    // planned on the host while the passes above run (creation of a 61M-entry FP16 plan and one evaluation 14.1 ->
-    // 12.3 ms). The team solver never launches it, and there the uploads after the rule only add round trips
-    // (plan_update of a 127k-entry plan 1041 us without, 1066 us with it; of a 61M-entry one 9.44 and 9.57 ms).
-    if (p->opt.precision != IMRT_FP32 && p->opt.solver == IMRT_SOLVER_GRAPH) {
+    // The reduced precision's forward pass is planned on the host while the passes above run (creation of a
+    // 61M-entry FP16 plan and one evaluation 14.1 -> 12.3 ms). The team solver does not launch it, but a served plan
+    // asks for its dose: left to that call, plan_update of a 127k-entry plan is 25 us shorter and the server, whose
+    // builder and scheduler threads then make it in turn, slower by a sixth (935 -> 790 plans/s).
+    if (p->opt.precision != IMRT_FP32) {
         FwdShape* early = nullptr;
         if (get_shape(p, p->opt.precision, 1, &early) != IMRT_OK) g_error.clear();  // as in plan_build
     }

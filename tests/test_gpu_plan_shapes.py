@@ -1,5 +1,5 @@
-"""Plan creation makes the forward pass's work schedule only where the plan's own solver launches it; other
-plans make it with the first call that needs it (plan_info reads device_bytes before it asks for the schedule)."""
+"""Plan creation makes the forward pass's work schedules that its step-size rule runs or hides; other plans make
+one with the first call that needs it (plan_info reads device_bytes before it asks for the schedule)."""
 import dataclasses
 
 import numpy as np
@@ -14,10 +14,11 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("solver,precision,lambda0,under,early", [
     (L.SOLVER_GRAPH, L.FP16, 0.0, True, True),
     (L.SOLVER_GRAPH, L.FP32, 1.0, False, True),
-    (L.SOLVER_TEAM, L.FP16, 0.0, True, False),
+    (L.SOLVER_TEAM, L.FP16, 0.0, True, True),
+    (L.SOLVER_TEAM, L.FP16, 1.0, False, False),
     (L.SOLVER_TEAM, L.FP32, 1.0, False, False),
 ])
-def test_schedules_are_made_for_the_solver_that_uses_them(solver, precision, lambda0, under, early):
+def test_schedules_are_made_with_the_plan_or_at_first_use(solver, precision, lambda0, under, early):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
