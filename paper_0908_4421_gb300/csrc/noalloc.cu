@@ -496,6 +496,7 @@ extern "C" imrt_status imrt_eval_csr_noalloc(const imrt_csr* D, const uint8_t* s
     const int blocks = n_tiles < sms * kNaBlocksPerSm ? n_tiles : sms * kNaBlocksPerSm;
     const int want = (D->m + 8 * kNaThreads - 1) / (8 * kNaThreads);
     const int count_blocks = want < kNaCountBlocks ? want : kNaCountBlocks;
+    const bool copy_G = needs_copy(G_out);  // an objective wanted in device memory takes a copy of its own
     NaResult out{};
     if (e == cudaSuccess) {
         k_na_counts<<<count_blocks, kNaThreads, 0, cs>>>(structures, D->m, s);
@@ -514,8 +515,7 @@ extern "C" imrt_status imrt_eval_csr_noalloc(const imrt_csr* D, const uint8_t* s
         e = cudaLaunchKernelEx(&cfg, k_na_eval, D->row_ptr, D->col_idx, D->val, D->m, D->n, D->nnz, structures,
                                terms, x, z_out, tile_rows, n_tiles, count_blocks, s);
     }
-    // the objective and the error flag in one copy; an objective wanted in device memory takes a copy of its own
-    const bool copy_G = needs_copy(G_out);
+    // the objective and the error flag in one copy
     if (e == cudaSuccess) e = cudaMemcpyAsync(&out, &s->res, sizeof(out), cudaMemcpyDeviceToHost, cs);
     if (e == cudaSuccess && copy_G) e = cudaMemcpyAsync(G_out, &s->res.G, sizeof(double), cudaMemcpyDefault, cs);
     if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
