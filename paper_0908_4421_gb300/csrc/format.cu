@@ -307,13 +307,12 @@ __device__ __forceinline__ void store_t(const TDest& o, int64_t k, float v, int3
 
 // Pass 3: scatter, 32 voxel rows at a time in the caller's voxel order (it keeps a beamlet's voxels close
 // together in r, which the transposed pass gathers; the SELL permutation scatters them inside each sorting
-// window). Step a: every entry of the block's rows sets its row's bit in its beamlet's mask. Step b: an entry's position in its
-// beamlet row is the beamlet's cursor plus the number of the block's lower rows holding that
-// beamlet (the mask bits below its own), so each beamlet row still receives its voxels in
-// ascending index, with no ordering between the threads. Step c: each cursor advances by its
-// mask's population and the masks are cleared. A warp takes whole rows (coalesced loads, eight
-// in flight per lane). (Splitting the launch into beamlet ranges whose writes stay in L2 was
-// measured slower: every range re-reads the column indices.)
+// window). Step a: every entry of the block's rows sets its row's bit in its beamlet's mask. Step b: an entry's
+// position in its beamlet row is the beamlet's cursor plus the number of the block's lower rows holding that
+// beamlet (the mask bits below its own), so each beamlet row receives its voxels in ascending index, with no
+// ordering between the threads. Step c: each cursor advances by its mask's population and the masks are cleared. A
+// warp takes whole rows (coalesced loads, eight in flight per lane). (Splitting the launch into beamlet ranges whose
+// writes stay in L2 was measured slower: every range re-reads the column indices.)
 constexpr int kTBlockRows = 32;
 template <bool PAIR>
 __global__ void k_t_scatter(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
