@@ -652,6 +652,7 @@ imrt_status finish_shape(imrt_plan* p, const SellCopy& c, int variant, FwdShape*
         int64_t* tab = nullptr;
         TRY(dalloc(p, &tab, (size_t)2 * count));
         CK(launch_prefetch_table(p->bwd_order, p->t_seg, p->t_H, p->n, count, cap, tab, stream_of(p)));
+        CK(cudaStreamSynchronize(stream_of(p)));  // a later call may run on another stream (plan_set_options)
         out->pf_tab = tab;
         out->pf_per_cta = per_cta;
     }
