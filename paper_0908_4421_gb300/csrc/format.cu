@@ -448,15 +448,15 @@ __global__ void __launch_bounds__(256) k_tq_fill(const int64_t* __restrict__ t_o
         const int64_t f = src[h] + (ps - sb[h]) + ((e - ps) >> 3);
         float v[8];
         uint32_t lo[8];
-        // a padding entry (value 0) names the run's last voxel: r is written there in every pass, which it is
-        // not at voxels without entries
-        const uint32_t pad = f + 7 * sg < src[h + 1] ? 0u : __ldg(pair + src[h + 1] - 1).y;
+        // a padding entry (value 0) names the voxel of its group's first entry, which is never padding (a piece
+        // of sg groups has more than 8 (sg - 1) entries): r of a voxel with entries is written in every pass, r
+        // of one without is not
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
             const bool in = f + t * sg < src[h + 1];
-            const uint2 w = in ? __ldg(pair + f + t * sg) : make_uint2(0u, pad);
+            const uint2 w = in ? __ldg(pair + f + t * sg) : make_uint2(0u, 0u);
             v[t] = __uint_as_float(w.x);
-            lo[t] = w.y & 0xffffu;
+            lo[t] = in ? w.y & 0xffffu : (t ? lo[0] : 0u);
         }
         float4* sv = reinterpret_cast<float4*>(s_val + e);
         sv[0] = make_float4(v[0], v[1], v[2], v[3]);
