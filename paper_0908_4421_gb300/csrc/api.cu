@@ -652,7 +652,6 @@ imrt_status finish_shape(imrt_plan* p, const SellCopy& c, int variant, FwdShape*
         int64_t* tab = nullptr;
         TRY(dalloc(p, &tab, (size_t)2 * count));
         CK(launch_prefetch_table(p->bwd_order, p->t_seg, p->t_H, p->n, count, cap, tab, stream_of(p)));
-        CK(cudaStreamSynchronize(stream_of(p)));  // a later call may run on another stream (plan_set_options)
         out->pf_tab = tab;
         out->pf_per_cta = per_cta;
     }
@@ -2490,6 +2489,9 @@ imrt_status plan_info(const imrt_plan* pc, imrt_plan_info* info) {
         info->fwd_schedule = sh->variant == 1 ? 1 : (sh->units.local ? 0 : 2);
         info->fwd_units = sh->units.n_units;
     }
+    // what this call prepared is complete before a later one reads it on another stream (plan_set_options); every
+    // other call that prepares a schedule ends with such a wait
+    CK(cudaStreamSynchronize(stream_of(p)));
     info->bwd_grid = p->bwd_grid;
     info->bwd_block = kBwdThreads;
     info->precision = p->opt.precision;
