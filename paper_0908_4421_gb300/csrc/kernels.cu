@@ -487,8 +487,9 @@ __device__ __forceinline__ void power_next_x(const float* __restrict__ w, int n,
     for (int k = 0; k < kWarps; ++k) most = max(most, part_m[k]);
     const uint32_t ex = min(max(most >> 23, 1u), 253u);          // max |w| < 2^(ex - 126), or 2^128
     const float scale = __uint_as_float((254u - ex) << 23);      // 2^(127 - ex)
-    WideSum ww{0.0f, 0.0f, 0.0f};
-    for (int i = tid; i < n_pad; i += kFwdThreads) ww = wide_add(ww, wide_square(xs[i] * scale));  // this thread's entries
+    WideSum ww{0.0f, 0.0f, 0.0f};  // this thread's entries
+    if (tid < n_pad) ww = wide_square(xs[tid] * scale);
+    for (int i = tid + kFwdThreads; i < n_pad; i += kFwdThreads) ww = wide_add(ww, wide_square(xs[i] * scale));
     ww = warp_sum(ww, 16);
     if (lane == 0) part[wib] = ww;
     __syncthreads();
